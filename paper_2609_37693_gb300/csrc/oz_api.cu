@@ -119,9 +119,10 @@ oz_status dgemm_run(oz_plan plan, int trans_a, int trans_b, int64_t m, int64_t n
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   char* ws = static_cast<char*>(workspace);
   int32_t* flag = reinterpret_cast<int32_t*>(ws + L.flag);
-  cudaError_t e = cudaMemsetAsync(flag, 0, 16, st);
-  if (e != cudaSuccess) return OZ_ERR_CUDA;
-  if (k == 0) return cuda_status(cudaMemset2DAsync(C, (size_t)ldc * 8, 0, (size_t)n * 8, (size_t)m, st));
+  if (k == 0) {
+    cudaError_t z = cudaMemsetAsync(flag, 0, 16, st);
+    return cuda_status(z == cudaSuccess ? cudaMemset2DAsync(C, (size_t)ldc * 8, 0, (size_t)n * 8, (size_t)m, st) : z);
+  }
 
   const OzTables& T = plan->tab;
   const int bf16 = oz::engine_bf16(plan->engine);
@@ -132,6 +133,9 @@ oz_status dgemm_run(oz_plan plan, int trans_a, int trans_b, int64_t m, int64_t n
   void* V = ws + L.v;
   uint8_t* Y = reinterpret_cast<uint8_t*>(ws + L.y);
 
+  // bf16 planes: both operands split together; the launch clears the status word itself
+  cudaError_t e = bf16 ? cudaSuccess : cudaMemsetAsync(flag, 0, 16, st);
+  if (e != cudaSuccess) return OZ_ERR_CUDA;
   if (plan->is_fp) {
     if (!plan->d_words) return OZ_ERR_CUDA;
     const OzFpTables& F = plan->fp;
@@ -146,34 +150,38 @@ oz_status dgemm_run(oz_plan plan, int trans_a, int trans_b, int64_t m, int64_t n
     if (e != cudaSuccess) return OZ_ERR_CUDA;
     return cuda_status(oz::launch_reconstruct16(T, m, n, Y16, L.ldy, s, t, C, ldc, st));
   }
-  // Scale + Reduce, A side: vectors are the rows of op(A).
-  e = trans_a ? oz::launch_split_cols(T, m, k, A, lda, L.m_pad, L.k_pad, s, U, bf16, flag, colmax, st)
-              : oz::launch_split_rows(T, m, k, A, lda, L.m_pad, L.k_pad, s, U, bf16, flag, st);
-  if (e != cudaSuccess) return OZ_ERR_CUDA;
-  // B side: vectors are the columns of op(B). Bf16 planes are split from
-  // B's columns in place (column maxima, then tiles staged through shared
-  // memory); for int8 planes B (k x n) is transposed first, so that its
-  // columns are split as contiguous rows.
-  if (trans_b) {
-    e = oz::launch_split_rows(T, n, k, B, ldb, L.n_pad, L.k_pad, t, V, bf16, flag, st);
-  } else if (bf16) {
-    e = oz::launch_split_cols(T, n, k, B, ldb, L.n_pad, L.k_pad, t, V, bf16, flag, colmax, st);
+  // Scale + Reduce: the vectors of the A side are the rows of op(A), those of
+  // the B side the columns of op(B). Bf16 planes are split from strided
+  // columns in place (A's column maxima go where Y will be, at least 16 bytes
+  // a row); for int8 planes B (k x n) is transposed first, so that its columns
+  // are split as contiguous rows.
+  if (bf16) {
+    const oz::SplitOperand oa = {!trans_a, A, lda, m, L.m_pad, s, U, reinterpret_cast<uint64_t*>(Y)};
+    const oz::SplitOperand ob = {trans_b != 0, B, ldb, n, L.n_pad, t, V, colmax};
+    e = oz::launch_split_both(T, oa, ob, k, L.k_pad, flag, st);
   } else {
-    double* Bt = reinterpret_cast<double*>(ws + L.bt);
-    e = oz::launch_transpose(k, n, B, ldb, Bt, st);
-    if (e == cudaSuccess) e = oz::launch_split_rows(T, n, k, Bt, k, L.n_pad, L.k_pad, t, V, bf16, flag, st);
+    e = trans_a ? oz::launch_split_cols(T, m, k, A, lda, L.m_pad, L.k_pad, s, U, bf16, flag, colmax, st)
+                : oz::launch_split_rows(T, m, k, A, lda, L.m_pad, L.k_pad, s, U, bf16, flag, st);
+    if (e == cudaSuccess && trans_b) {
+      e = oz::launch_split_rows(T, n, k, B, ldb, L.n_pad, L.k_pad, t, V, bf16, flag, st);
+    } else if (e == cudaSuccess) {
+      double* Bt = reinterpret_cast<double*>(ws + L.bt);
+      e = oz::launch_transpose(k, n, B, ldb, Bt, st);
+      if (e == cudaSuccess) e = oz::launch_split_rows(T, n, k, Bt, k, L.n_pad, L.k_pad, t, V, bf16, flag, st);
+    }
   }
   if (e != cudaSuccess) return OZ_ERR_CUDA;
   // GEMMs + epilogue; with too few output tiles, the inner dimension split into
   // ranges whose residue sets are then added modulo m (the layout's split: a
   // TC plan forced onto one CTA per tile runs unsplit)
+  const oz::MarkedShifts marks = bf16 ? oz::MarkedShifts{s, t} : oz::MarkedShifts{nullptr, nullptr};
   const bool forced_single = single_cta && plan->engine == OZ_ENGINE_TC;
   const oz::KSplit split = forced_single ? oz::KSplit{1, 0} : L.split;
   e = (plan->engine == OZ_ENGINE_TC1 || forced_single)
           ? oz::launch_gemm_tc_single(T, m, n, L.m_pad, L.n_pad, L.k_pad, U, V, Y, L.ldy, 0, flag, st, split,
-                                      (int64_t)L.ysplit)
+                                      (int64_t)L.ysplit, marks)
       : bf16 ? oz::launch_gemm_tc(T, m, n, L.m_pad, L.n_pad, L.k_pad, U, V, Y, L.ldy, 0, flag, st, split,
-                                  (int64_t)L.ysplit)
+                                  (int64_t)L.ysplit, marks)
              : oz::launch_gemm_imma(T, m, n, L.k_pad, static_cast<const int8_t*>(U), L.m_pad * L.k_pad,
                                     static_cast<const int8_t*>(V), L.n_pad * L.k_pad, Y, L.ldy, 0, st);
   if (e != cudaSuccess) return OZ_ERR_CUDA;

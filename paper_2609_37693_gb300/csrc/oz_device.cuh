@@ -17,6 +17,42 @@ static __device__ __forceinline__ int32_t shift_from_maxbits(uint64_t mb, int be
   return beta - e;
 }
 
+// Programmatic dependent launch: a kernel launched by launch_pdl (oz_launch.h)
+// may start while the kernel before it on the stream is still running. Every
+// kernel of a product therefore waits here, before its first access to global
+// memory, until that kernel has finished and its writes are visible, and then
+// lets its own successor be scheduled. Both are no-ops after a plain launch.
+static __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+static __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// A load of what an earlier kernel of the stream may have written: an ordinary
+// one, which stays below pdl_wait. (ld.global.nc wants its data unwritten for
+// the kernel's whole life, part of which a dependent launch spends beside its
+// predecessor; so no __ldg, and no const __restrict__ kernel parameter.)
+template <typename T>
+static __device__ __forceinline__ T ld_dep(const T* p) {
+  return *p;
+}
+
+// The mark of a vector that holds a non-finite entry: oz_dgemm's split adds it
+// to the vector's shift (shifts lie within about +-1200), and the GEMM
+// kernel takes it off again and sets bit 0 of the status word. The split can
+// so clear the status word itself instead of a memset ahead of it.
+constexpr int32_t kBadMark = 1 << 24;
+
+// Thread `tid` of `threads`: unmark the shifts of both operands.
+static __device__ __forceinline__ void unmark_shifts(int32_t* __restrict__ s, int m, int32_t* __restrict__ t, int n,
+                                                     int32_t* status, int tid, int threads) {
+  for (int i = tid; i < m + n; i += threads) {
+    int32_t* p = i < m ? s + i : t + (i - m);
+    const int32_t v = *p;
+    if (v > kBadMark / 2) {
+      *p = v - kBadMark;
+      atomicOr(status, 1);
+    }
+  }
+}
+
 // Decoded truncated integer of one entry: |a'| and its sign.
 struct Trunc {
   uint64_t mag;

@@ -41,6 +41,7 @@
 #include "oz_sync.cuh"
 #include "oz_pair.cuh"
 #include "oz_device.cuh"
+#include "oz_launch.h"
 
 namespace oz {
 namespace {
@@ -307,6 +308,11 @@ struct Params {
   // writes its digits to Y + j ysplit
   int nsplit, kbps;
   int64_t ysplit;
+  MarkedShifts marks;
+  // Epilogue thread tid of `threads` (all CTAs): unmark the shifts
+  __device__ __forceinline__ void unmark(int tid, int threads) const {
+    if (marks.s) unmark_shifts(marks.s, m, marks.t, n, status, tid, threads);
+  }
 };
 
 // The tile, split and k-block range [kb0, kb1) of unit u.
@@ -369,6 +375,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_holder;
+  pdl_wait();
+  pdl_trigger();
 
   const int num_units = p.num_tiles * p.nsplit;
 
@@ -448,6 +456,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     const int quarter = warp & 3;            // TMEM lanes 32*quarter .. +31
     const int cbase = (e >> 2) * CPW1;       // columns cbase .. cbase + CPW1 - 1
     const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
+    p.unmark(blockIdx.x * (kEpiWarps * 32) + threadIdx.x - 64, gridDim.x * (kEpiWarps * 32));
     uint32_t g = 0;
     bool ok = true;
     for (int t = blockIdx.x; t < num_units && ok; t += gridDim.x) {
@@ -561,6 +570,7 @@ struct PairSingle {
   __device__ __forceinline__ int units() const { return p.num_tiles * p.nsplit; }
   __device__ __forceinline__ int32_t* status() const { return p.status; }
   __device__ __forceinline__ int first(int) const { return 0; }
+  __device__ __forceinline__ void unmark(int tid, int threads) const { p.unmark(tid, threads); }
   __device__ __forceinline__ void prefetch() const {
     asm volatile("prefetch.tensormap [%0];" ::"l"(&mapA) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&mapB) : "memory");
@@ -603,6 +613,7 @@ struct PairGrouped {
     return group_find(probs, count, (int64_t)(t < total ? t : 0), [](const OzGroupProblem& q) { return q.unit_begin; });
   }
   __device__ __forceinline__ void prefetch() const {}
+  __device__ __forceinline__ void unmark(int, int) const {}
   __device__ __forceinline__ PairUnit unit(int t, int& pi) const {
     while (pi + 1 < count && probs[pi + 1].unit_begin <= t) ++pi;
     const OzGroupProblem& P = probs[pi];
@@ -679,6 +690,8 @@ gemm_tc_pair_kernel(const __grid_constant__ S sched, const __grid_constant__ OzT
   cluster_sync();                           // both CTAs' barriers exist before any remote use
   tc_fence_after();
   const uint32_t tmem_base = *tmem_holder;
+  pdl_wait();
+  pdl_trigger();
 
   const int num_units = sched.units();
   int32_t* const status = sched.status();
@@ -767,6 +780,7 @@ gemm_tc_pair_kernel(const __grid_constant__ S sched, const __grid_constant__ OzT
     const int quarter = warp & 3;
     const int cbase = (e >> 2) * CPW;          // first column this warp drains
     const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
+    sched.unmark((int)blockIdx.x * (EW * 32) + (int)threadIdx.x - 64, (int)gridDim.x * (EW * 32));
     uint32_t g = 0;
     bool ok = true;
     int pi = sched.first(pair);
@@ -1086,7 +1100,7 @@ bool set_split(Params* p, KSplit split, int64_t ysplit) {
 
 cudaError_t launch_gemm_tc(const OzTables& t, int64_t m, int64_t n, int64_t m_pad, int64_t n_pad, int64_t k_pad,
                            const void* U, const void* V, uint8_t* Y, int64_t ldy, int raw, int32_t* status,
-                           cudaStream_t st, KSplit split, int64_t ysplit) {
+                           cudaStream_t st, KSplit split, int64_t ysplit, MarkedShifts marks) {
   if (m == 0 || n == 0) return cudaSuccess;
   if (ldy < n) return cudaErrorInvalidValue;
   // pair tiles: 256 x 256 per CTA pair
@@ -1137,11 +1151,11 @@ cudaError_t launch_gemm_tc(const OzTables& t, int64_t m, int64_t n, int64_t m_pa
   p.Y = Y;
   p.ldy = ldy;
   p.status = status;
+  p.marks = marks;
   if (!set_split(&p, split, ysplit)) return cudaErrorInvalidValue;
   const int64_t units = num_tiles * p.nsplit;
   const int64_t pairs = units < sms / 2 ? units : sms / 2;
-  kernel<<<(unsigned)(2 * pairs), (2 + epi_warps) * 32, smem_bytes, st>>>(sched, t);
-  return cudaGetLastError();
+  return launch_pdl(kernel, dim3((unsigned)(2 * pairs)), dim3((2 + epi_warps) * 32), (size_t)smem_bytes, st, 1, sched, t);
 }
 
 // Tensor maps of one grouped problem's planes (rows of Q planes): 128-row
@@ -1191,7 +1205,8 @@ cudaError_t launch_gemm_tc_grouped(const OzTables& t, const OzGroupProblem* prob
 // The one-CTA kernel (128 x 256 tiles), kept for comparison.
 cudaError_t launch_gemm_tc_single(const OzTables& t, int64_t m, int64_t n, int64_t m_pad, int64_t n_pad,
                                   int64_t k_pad, const void* U, const void* V, uint8_t* Y, int64_t ldy, int raw,
-                                  int32_t* status, cudaStream_t st, KSplit split, int64_t ysplit) {
+                                  int32_t* status, cudaStream_t st, KSplit split, int64_t ysplit,
+                                  MarkedShifts marks) {
   if (m == 0 || n == 0) return cudaSuccess;
   if (ldy < n) return cudaErrorInvalidValue;
   if ((reinterpret_cast<uintptr_t>(U) & 127) || (reinterpret_cast<uintptr_t>(V) & 127) || k_pad % BK ||
@@ -1227,11 +1242,11 @@ cudaError_t launch_gemm_tc_single(const OzTables& t, int64_t m, int64_t n, int64
   p.Y = Y;
   p.ldy = ldy;
   p.status = status;
+  p.marks = marks;
   if (!set_split(&p, split, ysplit)) return cudaErrorInvalidValue;
   const int64_t units = num_tiles * p.nsplit;
   const int grid = (int)(units < sms ? units : sms);
-  kernel<<<grid, kThreads, kSmemBytes, st>>>(mapA, mapB, t, p);
-  return cudaGetLastError();
+  return launch_pdl(kernel, dim3((unsigned)grid), dim3(kThreads), (size_t)kSmemBytes, st, 1, mapA, mapB, t, p);
 }
 
 }  // namespace oz

@@ -214,6 +214,24 @@ cudaError_t launch_split_rows(const OzTables& t, int64_t nvec, int64_t len, cons
 cudaError_t launch_split_cols(const OzTables& t, int64_t nvec, int64_t len, const double* X, int64_t ld,
                               int64_t nvec_pad, int64_t k_pad, int32_t* shifts, void* planes, int bf16,
                               int32_t* flag, uint64_t* colmax, cudaStream_t st, bool given = false);
+// Both operands' shifts and bf16 planes in one or two launches, which also
+// clear the status word; vectors with a non-finite entry get a marked shift (kBadMark)
+// that the TC GEMM kernels unmark and report (their shifts argument).
+struct SplitOperand {
+  bool contiguous;       // vectors are rows of X (else its columns)
+  const double* X;
+  int64_t ld, nvec, nvec_pad;
+  int32_t* shifts;
+  void* planes;
+  uint64_t* colmax;      // scratch of nvec words, for columns (each operand its own)
+};
+cudaError_t launch_split_both(const OzTables& t, const SplitOperand& A, const SplitOperand& B, int64_t len,
+                              int64_t k_pad, int32_t* status, cudaStream_t st);
+// The shifts of both operands as launch_split_both left them (s of m rows, t
+// of n columns), for the GEMM to unmark; null: nothing to unmark.
+struct MarkedShifts {
+  int32_t *s, *t;
+};
 cudaError_t launch_gemm_imma(const OzTables& t, int64_t m, int64_t n, int64_t k_pad, const int8_t* U,
                              int64_t u_plane, const int8_t* V, int64_t v_plane, uint8_t* Y, int64_t ldy, int raw,
                              cudaStream_t st);
@@ -221,10 +239,12 @@ cudaError_t launch_gemm_imma(const OzTables& t, int64_t m, int64_t n, int64_t k_
 // split: the ranges of ksplit_for (nsplit 1: none), digit set j at Y + j ysplit
 cudaError_t launch_gemm_tc(const OzTables& t, int64_t m, int64_t n, int64_t m_pad, int64_t n_pad, int64_t k_pad,
                            const void* U, const void* V, uint8_t* Y, int64_t ldy, int raw, int32_t* status,
-                           cudaStream_t st, KSplit split = {1, 0}, int64_t ysplit = 0);
+                           cudaStream_t st, KSplit split = {1, 0}, int64_t ysplit = 0,
+                           MarkedShifts marks = {nullptr, nullptr});
 cudaError_t launch_gemm_tc_single(const OzTables& t, int64_t m, int64_t n, int64_t m_pad, int64_t n_pad, int64_t k_pad,
                            const void* U, const void* V, uint8_t* Y, int64_t ldy, int raw, int32_t* status,
-                           cudaStream_t st, KSplit split = {1, 0}, int64_t ysplit = 0);
+                           cudaStream_t st, KSplit split = {1, 0}, int64_t ysplit = 0,
+                           MarkedShifts marks = {nullptr, nullptr});
 // Y[0] = sum of the nsplit digit sets Y[j] (at Y + j ysplit) modulo each
 // modulus, over Q planes of m rows of ldy bytes (ldy a multiple of 16)
 cudaError_t launch_combine_digits(const OzTables& t, int64_t m, int64_t ldy, uint8_t* Y, int nsplit, int64_t ysplit,

@@ -39,6 +39,7 @@
 
 #include "oz_internal.h"
 #include "oz_device.cuh"
+#include "oz_launch.h"
 
 namespace oz {
 namespace {
@@ -597,16 +598,16 @@ __device__ __forceinline__ void fill_kP(const OzTables& T, uint4* kP) {
 // thread holds in its shared-memory slots wsm[q * QS].
 template <int NT, int NP2, int NQ4, int QS = 256>
 __device__ __forceinline__ void rec4_groups(const OzTables& T, const uint4* kP, const uint32_t* wsm, int64_t i,
-                                            int64_t j0, int64_t n, int32_t si, const int32_t* __restrict__ t,
+                                            int64_t j0, int64_t n, int32_t si, const int32_t* t,
                                             double* __restrict__ C, int64_t ldc) {
   constexpr int Q = 3 * NT + 2 * NP2 + 4 * NQ4;
   int32_t tj[4];
   if (j0 + 4 <= n && (reinterpret_cast<uintptr_t>(t + j0) & 15) == 0) {
-    const int4 v = __ldg(reinterpret_cast<const int4*>(t + j0));
+    const int4 v = ld_dep(reinterpret_cast<const int4*>(t + j0));
     tj[0] = v.x, tj[1] = v.y, tj[2] = v.z, tj[3] = v.w;
   } else {
 #pragma unroll
-    for (int e = 0; e < 4; ++e) tj[e] = j0 + e < n ? __ldg(t + j0 + e) : 0;
+    for (int e = 0; e < 4; ++e) tj[e] = j0 + e < n ? ld_dep(t + j0 + e) : 0;
   }
   uint32_t w[Q];
 #pragma unroll
@@ -693,8 +694,8 @@ __device__ __forceinline__ void issue_digits8(const uint8_t* __restrict__ Y, int
 template <int NT, int NP2, int NQ4>
 __global__ void __launch_bounds__(256, 2) reconstruct_groups_kernel(const __grid_constant__ OzTables T, int64_t m,
                                                                     int64_t n, const uint8_t* __restrict__ Y,
-                                                                    int64_t ldy, const int32_t* __restrict__ s,
-                                                                    const int32_t* __restrict__ t,
+                                                                    int64_t ldy, const int32_t* s,
+                                                                    const int32_t* t,
                                                                     double* __restrict__ C, int64_t ldc,
                                                                     int64_t nch, int tpr_log2) {
   constexpr int Q = 3 * NT + 2 * NP2 + 4 * NQ4;
@@ -702,6 +703,8 @@ __global__ void __launch_bounds__(256, 2) reconstruct_groups_kernel(const __grid
   __shared__ uint32_t buf[2][Q * 256];
   fill_kP(T, kP);
   __syncthreads();
+  pdl_wait();
+  pdl_trigger();
   const int tpr = 1 << tpr_log2, rows = 256 >> tpr_log2;
   const int r_in = threadIdx.x >> tpr_log2, c_in = threadIdx.x & (tpr - 1);
   const int64_t plane = m * ldy;
@@ -721,7 +724,7 @@ __global__ void __launch_bounds__(256, 2) reconstruct_groups_kernel(const __grid
     cp_async_commit();
     cp_async_wait1();                       // this task's copies have landed
     const int64_t i = row_of(gi), j0 = col_of(c);
-    if (i < m && j0 < n) rec4_groups<NT, NP2, NQ4>(T, kP, mine + slot * Q * 256, i, j0, n, __ldg(s + i), t, C, ldc);
+    if (i < m && j0 < n) rec4_groups<NT, NP2, NQ4>(T, kP, mine + slot * Q * 256, i, j0, n, ld_dep(s + i), t, C, ldc);
     slot ^= 1;
     b = bn, gi = gn, c = cn;
   }
@@ -734,8 +737,8 @@ __global__ void __launch_bounds__(256, 2) reconstruct_groups_kernel(const __grid
 template <int NT, int NP2, int NQ4>
 __global__ void __launch_bounds__(256, 2) reconstruct_groups8_kernel(const __grid_constant__ OzTables T, int64_t m,
                                                                      int64_t n, const uint8_t* __restrict__ Y,
-                                                                     int64_t ldy, const int32_t* __restrict__ s,
-                                                                     const int32_t* __restrict__ t,
+                                                                     int64_t ldy, const int32_t* s,
+                                                                     const int32_t* t,
                                                                      double* __restrict__ C, int64_t ldc,
                                                                      int64_t nch, int tpr_log2) {
   constexpr int Q = 3 * NT + 2 * NP2 + 4 * NQ4;
@@ -743,6 +746,8 @@ __global__ void __launch_bounds__(256, 2) reconstruct_groups8_kernel(const __gri
   extern __shared__ uint32_t dbuf[];
   fill_kP(T, kP);
   __syncthreads();
+  pdl_wait();
+  pdl_trigger();
   const int tpr = 1 << tpr_log2, rows = 256 >> tpr_log2;
   const int r_in = threadIdx.x >> tpr_log2, c_in = threadIdx.x & (tpr - 1);
   const int64_t plane = m * ldy;
@@ -764,7 +769,7 @@ __global__ void __launch_bounds__(256, 2) reconstruct_groups8_kernel(const __gri
     cp_async_wait1();                       // this task's copies have landed
     const int64_t i = row_of(gi), j0 = col_of(c);
     if (i < m && j0 < n) {
-      const int32_t si = __ldg(s + i);
+      const int32_t si = ld_dep(s + i);
       const uint32_t* w = mine + slot * Q * 512;
       rec4_groups<NT, NP2, NQ4, 512>(T, kP, w, i, j0, n, si, t, C, ldc);
       if (j0 + 4 < n) rec4_groups<NT, NP2, NQ4, 512>(T, kP, w + 1, i, j0 + 4, n, si, t, C, ldc);
@@ -874,17 +879,14 @@ cudaError_t launch_groups(const OzTables& T, int64_t m, int64_t n, const uint8_t
     cudaError_t e = cudaFuncSetAttribute(reconstruct_groups8_kernel<NT, NP2, NQ4>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    int per = 0, dev = 0, sms = 0;
+    int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, reconstruct_groups8_kernel<NT, NP2, NQ4>, 256, smem) !=
-            cudaSuccess)
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
       return cudaErrorInvalidValue;
-    int64_t grid = (int64_t)sms * (per > 0 ? per : 1);
+    int64_t grid = 2 * (int64_t)sms;                 // two blocks resident per SM (registers and digit buffers)
     if (grid > total) grid = total;
-    reconstruct_groups8_kernel<NT, NP2, NQ4><<<(unsigned)grid, 256, smem, st>>>(T, m, n, Y, ldy, s, t, C, ldc, nch,
-                                                                               tpr_log2);
-    return cudaGetLastError();
+    return launch_pdl(reconstruct_groups8_kernel<NT, NP2, NQ4>, dim3((unsigned)grid), dim3(256), (size_t)smem, st, 1, T,
+                      m, n, Y, ldy, s, t, C, ldc, nch, tpr_log2);
   }
   int tpr_log2 = 5;                                  // 32 .. 256 threads per row chunk of 4 tpr entries
   while (tpr_log2 < 8 && ((int64_t)4 << tpr_log2) < n) ++tpr_log2;

@@ -36,6 +36,9 @@
 
 #include "oz_internal.h"
 #include "oz_device.cuh"
+#include "oz_launch.h"
+#include "oz_pair.cuh"
+#include "oz_sync.cuh"
 
 namespace oz {
 namespace {
@@ -200,7 +203,7 @@ __device__ __forceinline__ void store_residues(const OzTables& T, const Pieces<N
 // and whether any of those entries is not finite: 16-byte loads (two
 // entries) when the row is 16-byte aligned, four of them in flight per
 // iteration, so that a short row's maximum is not a chain of load latencies.
-__device__ __forceinline__ void row_absmax(const uint64_t* __restrict__ row, int64_t len, int t, int step,
+__device__ __forceinline__ void row_absmax(const uint64_t* row, int64_t len, int t, int step,
                                            uint64_t& mx, uint32_t& bad) {
   auto fold = [&](uint64_t b) {
     b &= kAbsMask;
@@ -214,7 +217,7 @@ __device__ __forceinline__ void row_absmax(const uint64_t* __restrict__ row, int
     for (; p + 3 * (int64_t)step < np; p += 4 * (int64_t)step) {
       ulonglong2 v[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) v[u] = __ldg(r2 + p + u * step);
+      for (int u = 0; u < 4; ++u) v[u] = ld_dep(r2 + p + u * step);
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         fold(v[u].x);
@@ -222,13 +225,13 @@ __device__ __forceinline__ void row_absmax(const uint64_t* __restrict__ row, int
       }
     }
     for (; p < np; p += step) {
-      const ulonglong2 v = __ldg(r2 + p);
+      const ulonglong2 v = ld_dep(r2 + p);
       fold(v.x);
       fold(v.y);
     }
-    if ((len & 1) && t == 0) fold(__ldg(row + len - 1));
+    if ((len & 1) && t == 0) fold(ld_dep(row + len - 1));
   } else {
-    for (int64_t h = t; h < len; h += step) fold(__ldg(row + h));
+    for (int64_t h = t; h < len; h += step) fold(ld_dep(row + h));
   }
 }
 
@@ -236,7 +239,7 @@ template <bool kBF16, int NP, int QT>
 __device__ __forceinline__ void split_row(const OzTables& T, int64_t v, int64_t nvec, int64_t len,
                                           const double* __restrict__ X, int64_t ld, int64_t nvec_pad, int64_t k_pad,
                                           int32_t* __restrict__ shifts, void* __restrict__ planes,
-                                          int32_t* __restrict__ flag, bool given) {
+                                          int32_t* __restrict__ flag, bool given, bool mark = false) {
   __shared__ uint64_t red[8];
   __shared__ int32_t s_sh;
   const int tid = threadIdx.x;
@@ -264,7 +267,7 @@ __device__ __forceinline__ void split_row(const OzTables& T, int64_t v, int64_t 
       if (anybad && flag) atomicOr(flag, 1);
       int32_t s0 = live ? shift_from_maxbits(anybad ? 0 : m, T.bits) : 0;
       s_sh = s0;
-      if (live) shifts[v] = s0;
+      if (live) shifts[v] = s0 + (mark && anybad ? kBadMark : 0);
     }
     __syncthreads();
     s = s_sh;
@@ -278,13 +281,13 @@ __device__ __forceinline__ void split_row(const OzTables& T, int64_t v, int64_t 
     if (vec && h0 + 8 <= len) {
 #pragma unroll
       for (int e = 0; e < 8; e += 2) {
-        const ulonglong2 w = __ldg(reinterpret_cast<const ulonglong2*>(row + h0 + e));
+        const ulonglong2 w = ld_dep(reinterpret_cast<const ulonglong2*>(row + h0 + e));
         b[e] = w.x;
         b[e + 1] = w.y;
       }
     } else {
 #pragma unroll
-      for (int e = 0; e < 8; ++e) b[e] = (live && h0 + e < len) ? __ldg(row + h0 + e) : 0ull;
+      for (int e = 0; e < 8; ++e) b[e] = (live && h0 + e < len) ? ld_dep(row + h0 + e) : 0ull;
     }
     Pieces<NP> P[8];
 #pragma unroll
@@ -303,7 +306,8 @@ template <bool kBF16, int NP, int QT>
 __device__ __forceinline__ void split_row_warp(const OzTables& T, int64_t v, int64_t nvec, int64_t len,
                                                const double* __restrict__ X, int64_t ld, int64_t nvec_pad,
                                                int64_t k_pad, int32_t* __restrict__ shifts,
-                                               void* __restrict__ planes, int32_t* __restrict__ flag, bool given) {
+                                               void* __restrict__ planes, int32_t* __restrict__ flag, bool given,
+                                               bool mark = false) {
   const int lane = threadIdx.x & 31;
   const bool live = v < nvec;
   const uint64_t* row = reinterpret_cast<const uint64_t*>(X) + (live ? v * ld : 0);
@@ -319,7 +323,7 @@ __device__ __forceinline__ void split_row_warp(const OzTables& T, int64_t v, int
     s = live ? shift_from_maxbits(bad ? 0 : mx, T.bits) : 0;
     if (lane == 0) {
       if (bad && flag) atomicOr(flag, 1);
-      if (live) shifts[v] = s;
+      if (live) shifts[v] = s + (mark && bad ? kBadMark : 0);
     }
   }
   const int64_t plane = nvec_pad * k_pad;
@@ -329,13 +333,13 @@ __device__ __forceinline__ void split_row_warp(const OzTables& T, int64_t v, int
     if (vec && h0 + 8 <= len) {
 #pragma unroll
       for (int e = 0; e < 8; e += 2) {
-        const ulonglong2 w = __ldg(reinterpret_cast<const ulonglong2*>(row + h0 + e));
+        const ulonglong2 w = ld_dep(reinterpret_cast<const ulonglong2*>(row + h0 + e));
         b[e] = w.x;
         b[e + 1] = w.y;
       }
     } else {
 #pragma unroll
-      for (int e = 0; e < 8; ++e) b[e] = (live && h0 + e < len) ? __ldg(row + h0 + e) : 0ull;
+      for (int e = 0; e < 8; ++e) b[e] = (live && h0 + e < len) ? ld_dep(row + h0 + e) : 0ull;
     }
     Pieces<NP> P[8];
 #pragma unroll
@@ -396,12 +400,14 @@ __global__ void __launch_bounds__(256, (QT > 0 && NP == 4) ? 3 : 2) split_rows_g
 // Block (32 x 8): 32 consecutive columns, 8 warps over rows; each CTA covers
 // 256 rows.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void colmax_block(int64_t bx, int64_t by, int64_t nvec, int64_t len,
+// mark: a non-finite entry sets bit 63 of its column's word instead of the flag.
+__device__ __forceinline__ void colmax_block(int64_t bx, int64_t by, int tx, int ty, int64_t nvec, int64_t len,
                                              const double* __restrict__ X, int64_t ld,
-                                             uint64_t* __restrict__ colmax, int32_t* __restrict__ flag) {
+                                             uint64_t* __restrict__ colmax, int32_t* __restrict__ flag,
+                                             bool mark = false) {
   __shared__ uint64_t red[8][32];
-  const int64_t j = bx * 32 + threadIdx.x;
-  const int64_t h0 = by * 256 + threadIdx.y;
+  const int64_t j = bx * 32 + tx;
+  const int64_t h0 = by * 256 + ty;
   uint64_t mx = 0;
   uint32_t bad = 0;
   if (j < nvec) {
@@ -410,17 +416,17 @@ __device__ __forceinline__ void colmax_block(int64_t bx, int64_t by, int64_t nve
 #pragma unroll
     for (int i = 0; i < 32; ++i) {
       const int64_t h = h0 + 8 * i;
-      const uint64_t b = h < len ? __ldg(col + h * ld) & kAbsMask : 0ull;
+      const uint64_t b = h < len ? ld_dep(col + h * ld) & kAbsMask : 0ull;
       bad |= (uint32_t)((b >> 52) == 0x7ff);
       mx = b > mx ? b : mx;
     }
   }
   if (bad && flag) atomicOr(flag, 1);
-  red[threadIdx.y][threadIdx.x] = bad ? 0 : mx;
+  red[ty][tx] = bad ? (mark ? 1ull << 63 : 0ull) : mx;
   __syncthreads();
-  if (threadIdx.y == 0 && j < nvec) {
+  if (ty == 0 && j < nvec) {
     uint64_t m = 0;
-    for (int w = 0; w < 8; ++w) m = red[w][threadIdx.x] > m ? red[w][threadIdx.x] : m;
+    for (int w = 0; w < 8; ++w) m = red[w][tx] > m ? red[w][tx] : m;
     if (m) atomicMax(reinterpret_cast<unsigned long long*>(colmax + j), (unsigned long long)m);
   }
 }
@@ -428,7 +434,7 @@ __device__ __forceinline__ void colmax_block(int64_t bx, int64_t by, int64_t nve
 __global__ void __launch_bounds__(256) colmax_kernel(int64_t nvec, int64_t len, const double* __restrict__ X,
                                                      int64_t ld, uint64_t* __restrict__ colmax,
                                                      int32_t* __restrict__ flag) {
-  colmax_block(blockIdx.x, blockIdx.y, nvec, len, X, ld, colmax, flag);
+  colmax_block(blockIdx.x, blockIdx.y, threadIdx.x, threadIdx.y, nvec, len, X, ld, colmax, flag);
 }
 
 // Grouped: block b is block b - cm_begin of its problem's (ceil(n/32) x
@@ -438,7 +444,7 @@ __global__ void __launch_bounds__(256) colmax_grouped_kernel(const OzGroupProble
   const int64_t b = blockIdx.x;
   const OzGroupProblem& P = probs[__ldg(map + b)];
   const int64_t l = b - P.cm_begin, nbx = (P.n + 31) / 32;
-  colmax_block(l % nbx, l / nbx, P.n, P.k, P.B, P.ldb, P.colmax, P.flag);
+  colmax_block(l % nbx, l / nbx, threadIdx.x, threadIdx.y, P.n, P.k, P.B, P.ldb, P.colmax, P.flag);
 }
 
 __global__ void shifts_from_colmax_kernel(int64_t nvec, const uint64_t* __restrict__ colmax, int beta,
@@ -562,20 +568,19 @@ constexpr int kColTileJ = 32, kColTileH = 64;
 constexpr int kColPitchWords = 36;
 constexpr int kColPlaneWords = kColTileJ * kColPitchWords;     // 1152 words = 4608 bytes per modulus
 
-template <int NP, int QT>
-__device__ __forceinline__ void split_cols_tile(const OzTables& T, int64_t j0, int64_t hbase, int64_t nvec,
-                                                int64_t len, const double* __restrict__ X, int64_t ld,
-                                                int64_t nvec_pad, int64_t k_pad, const int32_t* __restrict__ shifts,
-                                                uint16_t* __restrict__ planes, uint32_t* tile) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int64_t j = j0 + lane;
-  const bool live = j < nvec;
-  const int32_t s = live ? __ldg(shifts + j) : 0;
-  const uint64_t* Xb = reinterpret_cast<const uint64_t*>(X);
-  const int64_t h0 = hbase + 8 * w;
-  uint64_t b[8];
+// Lane's eight entries of vector j at h0 .. h0 + 7 (zero past the operand).
+__device__ __forceinline__ void load_col8(const uint64_t* Xb, int64_t ld, bool live, int64_t j, int64_t h0,
+                                          int64_t len, uint64_t (&b)[8]) {
 #pragma unroll
-  for (int e = 0; e < 8; ++e) b[e] = (live && h0 + e < len) ? __ldg(Xb + (h0 + e) * ld + j) : 0ull;
+  for (int e = 0; e < 8; ++e) b[e] = (live && h0 + e < len) ? ld_dep(Xb + (h0 + e) * ld + j) : 0ull;
+}
+
+// One tile from the entries b of this thread (lane's vector, shift s).
+template <int NP, int QT>
+__device__ __forceinline__ void split_cols_entries(const OzTables& T, uint64_t (&b)[8], int32_t s, int64_t j0,
+                                                   int64_t hbase, int64_t nvec_pad, int64_t k_pad,
+                                                   uint16_t* __restrict__ planes, uint32_t* tile) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   Pieces<NP> P[8];
 #pragma unroll
   for (int e = 0; e < 8; ++e) {
@@ -608,6 +613,19 @@ __device__ __forceinline__ void split_cols_tile(const OzTables& T, int64_t j0, i
 }
 
 template <int NP, int QT>
+__device__ __forceinline__ void split_cols_tile(const OzTables& T, int64_t j0, int64_t hbase, int64_t nvec,
+                                                int64_t len, const double* __restrict__ X, int64_t ld,
+                                                int64_t nvec_pad, int64_t k_pad, const int32_t* __restrict__ shifts,
+                                                uint16_t* __restrict__ planes, uint32_t* tile) {
+  const int64_t j = j0 + (threadIdx.x & 31);
+  const bool live = j < nvec;
+  const int32_t s = live ? __ldg(shifts + j) : 0;
+  uint64_t b[8];
+  load_col8(reinterpret_cast<const uint64_t*>(X), ld, live, j, hbase + 8 * (threadIdx.x >> 5), len, b);
+  split_cols_entries<NP, QT>(T, b, s, j0, hbase, nvec_pad, k_pad, planes, tile);
+}
+
+template <int NP, int QT>
 __global__ void __launch_bounds__(256, 3) split_cols_bf16_kernel(const __grid_constant__ OzTables T, int64_t nvec,
                                                                 int64_t len, const double* __restrict__ X, int64_t ld,
                                                                 int64_t nvec_pad, int64_t k_pad,
@@ -630,6 +648,165 @@ __global__ void __launch_bounds__(256, 3) split_cols_grouped_kernel(const __grid
   const int64_t l = b - P.sc_begin, nbx = P.n_pad / kColTileJ;
   split_cols_tile<NP, QT>(T, (l % nbx) * kColTileJ, (l / nbx) * kColTileH, P.n, P.k, P.B, P.ldb, P.n_pad, P.k_pad,
                           P.t, static_cast<uint16_t*>(P.V), reinterpret_cast<uint32_t*>(col_tile));
+}
+
+// ---------------------------------------------------------------------------
+// Both operands of a product together (oz_dgemm, bf16 planes).
+//   Contiguous vectors: a block per row, or a warp per row when rows are
+//     short, as the kernels above.
+//   Strided vectors of at most kStripMaxK entries: a cluster of kStripCtas
+//     blocks per strip of 32 vectors. Block r of the cluster holds the strip's
+//     64-entry tiles r, r + kStripCtas, ...; it scans them for the maxima, the
+//     blocks exchange these through distributed shared memory, and each then
+//     splits its tiles (the last one from registers). No scratch, no second
+//     launch: 256^3 with the GEMM and the reconstruct in 28 us instead of 47.
+//   Longer strided vectors: a pass for the column maxima, then 32 x 64 tiles
+//     with the shifts formed from them. (A block's tiles of a strip would run
+//     one after another, with two barriers each: 189 us against 141 us at 4096.)
+// The maxima, strips and rows of a small product share one launch (most of
+// its time is launches and empty SMs); those of a large one are launched on
+// their own, since sharing costs them occupancy and L1 (the maxima run eight
+// blocks an SM alone and three beside the rows; the strips' staging buffers
+// shrink the rows' L1): 8192^3 560 us together, 519 us apart; 65536 x 256 rows
+// beside a 256 x 256 B 150 us against 121 us.
+// ---------------------------------------------------------------------------
+struct SplitSide {
+  const double* X;
+  int64_t ld, nvec, nvec_pad;
+  int32_t* shifts;
+  uint16_t* planes;
+  uint64_t* colmax;      // kSideTile: zeroed before the first launch
+  int kind;              // kSideRow, kSideWarp, kSideStrip or kSideTile
+  int blocks1, blocks2;  // rows, strips (a multiple of kStripCtas) or maxima; tiles
+};
+constexpr int kSideRow = 0, kSideWarp = 1, kSideStrip = 2, kSideTile = 3, kSideAny = -1;
+constexpr int kStripCtas = 8;
+constexpr int64_t kStripMaxK = 1024;
+
+template <int NP, int QT>
+__device__ __forceinline__ void split_strip(const OzTables& T, const SplitSide& S, int64_t strip, int64_t len,
+                                            int64_t k_pad, uint32_t* tile) {
+  __shared__ uint64_t red[8][32];
+  __shared__ uint64_t cmax[32];            // this block's column maxima, bit 63: a non-finite entry
+  __shared__ int32_t sh[32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const uint32_t rank = cluster_rank();
+  const int64_t j0 = strip * kColTileJ, j = j0 + lane;
+  const bool live = j < S.nvec;
+  const uint64_t* Xb = reinterpret_cast<const uint64_t*>(S.X);
+  const int ntiles = (int)(k_pad / kColTileH);
+  const int last = ntiles > (int)rank ? (int)rank + (ntiles - 1 - (int)rank) / kStripCtas * kStripCtas : -1;
+  uint64_t b[8];
+  uint64_t mx = 0, bad = 0;
+  for (int i = (int)rank; i < ntiles; i += kStripCtas) {
+    load_col8(Xb, S.ld, live, j, (int64_t)i * kColTileH + 8 * w, len, b);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const uint64_t a = b[e] & kAbsMask;
+      bad |= (uint64_t)((a >> 52) == 0x7ff) << 63;
+      mx = a > mx ? a : mx;
+    }
+  }
+  red[w][lane] = mx | bad;
+  __syncthreads();
+  if (w == 0) {
+    uint64_t m = 0, f = 0;
+#pragma unroll
+    for (int v = 0; v < 8; ++v) {
+      const uint64_t x = red[v][lane];
+      f |= x & ~kAbsMask;
+      m = (x & kAbsMask) > m ? (x & kAbsMask) : m;
+    }
+    cmax[lane] = m | f;
+  }
+  cluster_sync();
+  if (w == 0) {
+    uint64_t m = 0, f = 0;
+#pragma unroll
+    for (int r = 0; r < kStripCtas; ++r) {
+      uint64_t x;
+      asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(x) : "r"(mapa(smem_u32(&cmax[lane]), (uint32_t)r)) : "memory");
+      f |= x & ~kAbsMask;
+      m = (x & kAbsMask) > m ? (x & kAbsMask) : m;
+    }
+    const int32_t s = shift_from_maxbits(f ? 0 : m, T.bits);
+    sh[lane] = s;
+    if (rank == 0 && live) S.shifts[j] = s + (f ? kBadMark : 0);
+  }
+  __syncthreads();
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");   // done with the other blocks' maxima
+  const int32_t s = sh[lane];
+  for (int i = last; i >= 0; i -= kStripCtas) {
+    if (i != last) load_col8(Xb, S.ld, live, j, (int64_t)i * kColTileH + 8 * w, len, b);
+    split_cols_entries<NP, QT>(T, b, s, j0, (int64_t)i * kColTileH, S.nvec_pad, k_pad, S.planes, tile);
+    if (i >= kStripCtas) __syncthreads();            // the tile is read before the next one is staged
+  }
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");     // no block leaves while its maxima may be read
+}
+
+__device__ __forceinline__ void colmax_side(const SplitSide& S, int64_t l, int64_t len) {
+  const int64_t nbx = (S.nvec + 31) / 32;
+  colmax_block(l % nbx, l / nbx, threadIdx.x & 31, threadIdx.x >> 5, S.nvec, len, S.X, S.ld, S.colmax, nullptr, true);
+}
+
+// Blocks of side b, then side a (status: cleared, when not null).
+// KIND: the kind of every side, kSideRow or kSideWarp; kSideAny: each its own.
+template <int NP, int QT, int KIND>
+__global__ void __launch_bounds__(256, KIND == kSideAny && NP > 5 ? 2 : 3) split_both_kernel(
+    const __grid_constant__ OzTables T, const __grid_constant__ SplitSide a, const __grid_constant__ SplitSide b,
+    int64_t len, int64_t k_pad, int32_t* __restrict__ status) {
+  extern __shared__ uint4 col_tile[];
+  pdl_wait();
+  pdl_trigger();
+  if (status && blockIdx.x == 0 && threadIdx.x < 4) status[threadIdx.x] = 0;
+  const bool second = (int)blockIdx.x < b.blocks1;
+  const SplitSide& S = second ? b : a;
+  const int64_t l = second ? blockIdx.x : (int)blockIdx.x - b.blocks1;
+  const int kind = KIND == kSideAny ? S.kind : KIND;
+  if (kind == kSideStrip)
+    split_strip<NP, QT>(T, S, l / kStripCtas, len, k_pad, reinterpret_cast<uint32_t*>(col_tile));
+  else if (kind == kSideTile)
+    colmax_side(S, l, len);
+  else if (kind == kSideWarp)
+    split_row_warp<true, NP, QT>(T, l * 8 + (threadIdx.x >> 5), S.nvec, len, S.X, S.ld, S.nvec_pad, k_pad, S.shifts,
+                                 S.planes, nullptr, false, true);
+  else
+    split_row<true, NP, QT>(T, l, S.nvec, len, S.X, S.ld, S.nvec_pad, k_pad, S.shifts, S.planes, nullptr, false, true);
+}
+
+// The column maxima of the kSideTile sides.
+__global__ void __launch_bounds__(256) colmax_both_kernel(const __grid_constant__ SplitSide a,
+                                                          const __grid_constant__ SplitSide b, int64_t len,
+                                                          int32_t* __restrict__ status) {
+  pdl_wait();
+  pdl_trigger();
+  if (status && blockIdx.x == 0 && threadIdx.x < 4) status[threadIdx.x] = 0;
+  const bool second = (int)blockIdx.x < b.blocks1;
+  colmax_side(second ? b : a, second ? blockIdx.x : (int)blockIdx.x - b.blocks1, len);
+}
+
+// The tiles of the kSideTile sides, vectors fastest.
+template <int NP, int QT>
+__global__ void __launch_bounds__(256, NP > 5 ? 2 : 3) split_tiles_kernel(const __grid_constant__ OzTables T,
+                                                             const __grid_constant__ SplitSide a,
+                                                             const __grid_constant__ SplitSide b, int64_t len,
+                                                             int64_t k_pad) {
+  extern __shared__ uint4 col_tile[];
+  const bool second = (int)blockIdx.x < b.blocks2;
+  const SplitSide& S = second ? b : a;
+  const int l = second ? blockIdx.x : (int)blockIdx.x - b.blocks2;
+  const int nbx = (int)(S.nvec_pad / kColTileJ);
+  const int64_t j0 = (int64_t)(l % nbx) * kColTileJ, hbase = (int64_t)(l / nbx) * kColTileH;
+  const int64_t j = j0 + (threadIdx.x & 31);
+  const bool live = j < S.nvec;
+  pdl_wait();
+  pdl_trigger();
+  uint64_t v[8];
+  load_col8(reinterpret_cast<const uint64_t*>(S.X), S.ld, live, j, hbase + 8 * (threadIdx.x >> 5), len, v);
+  const uint64_t m = live ? ld_dep(S.colmax + j) : 0ull;
+  const int32_t s = shift_from_maxbits(m >> 63 ? 0ull : m, T.bits);
+  if (hbase == 0 && live && threadIdx.x < 32) S.shifts[j] = s + (m >> 63 ? kBadMark : 0);
+  split_cols_entries<NP, QT>(T, v, s, j0, hbase, S.nvec_pad, k_pad, S.planes, reinterpret_cast<uint32_t*>(col_tile));
 }
 
 // Transpose of a rows x cols block of doubles (row pitch ld) into cols x rows
@@ -715,6 +892,96 @@ cudaError_t split_cols_np(const OzTables& t, int64_t nvec, int64_t len, const do
 }
 
 }  // namespace
+
+namespace {
+
+// Entries of both operands up to which their passes share a launch.
+constexpr int64_t kMergeEntries = (int64_t)4 << 20;
+
+template <int NP, int QT>
+cudaError_t split_both_qt(const OzTables& t, const SplitSide& a, const SplitSide& b, int64_t len, int64_t k_pad,
+                          int32_t* status, cudaStream_t st) {
+  const int tile = t.Q * kColPlaneWords * 4;
+  for (auto kernel : {(const void*)split_both_kernel<NP, QT, kSideAny>, (const void*)split_tiles_kernel<NP, QT>}) {
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (QT > 0 ? QT : OZ_MAX_MODULI) * kColPlaneWords * 4);
+    if (e != cudaSuccess) return e;
+  }
+  for (const SplitSide* s : {&a, &b})
+    if (s->kind == kSideTile) {
+      cudaError_t e = cudaMemsetAsync(s->colmax, 0, 8 * (size_t)s->nvec, st);
+      if (e != cudaSuccess) return e;
+    }
+  auto rows = [](const SplitSide& s) { return s.kind == kSideRow || s.kind == kSideWarp; };
+  cudaError_t e = cudaSuccess;
+  // one launch of the sides x, y (either may be empty)
+  auto first = [&](SplitSide x, SplitSide y) {
+    if (e != cudaSuccess || x.blocks1 + y.blocks1 == 0) return;
+    const bool strips = (x.blocks1 && x.kind == kSideStrip) || (y.blocks1 && y.kind == kSideStrip);
+    const bool only_rows = (!x.blocks1 || rows(x)) && (!y.blocks1 || rows(y));   // then of one kind, by k_pad
+    e = launch_pdl(!only_rows ? split_both_kernel<NP, QT, kSideAny>
+                   : k_pad <= 1024 ? split_both_kernel<NP, QT, kSideWarp> : split_both_kernel<NP, QT, kSideRow>,
+                   dim3((unsigned)(x.blocks1 + y.blocks1)), dim3(256), strips ? (size_t)tile : 0, st,
+                   strips ? kStripCtas : 1, t, x, y, len, k_pad, status);
+    status = nullptr;
+  };
+  if ((a.nvec_pad + b.nvec_pad) * k_pad <= kMergeEntries || (rows(a) && rows(b))) {
+    first(a, b);
+  } else {
+    // the column maxima of both, then each operand's strips or rows
+    SplitSide none = {}, x = a, y = b;
+    if (x.kind != kSideTile) x.blocks1 = 0;
+    if (y.kind != kSideTile) y.blocks1 = 0;
+    if (x.blocks1 + y.blocks1 > 0) {
+      e = launch_pdl(colmax_both_kernel, dim3((unsigned)(x.blocks1 + y.blocks1)), dim3(256), 0, st, 1, x, y, len, status);
+      status = nullptr;
+    }
+    if (b.kind != kSideTile) first(none, b);
+    if (a.kind != kSideTile) first(a, none);
+  }
+  if (e != cudaSuccess || a.blocks2 + b.blocks2 == 0) return e;
+  return launch_pdl(split_tiles_kernel<NP, QT>, dim3((unsigned)(a.blocks2 + b.blocks2)), dim3(256), (size_t)tile, st, 1,
+                    t, a, b, len, k_pad);
+}
+
+SplitSide split_side(const SplitOperand& o, int64_t len, int64_t k_pad) {
+  SplitSide s = {};
+  s.X = o.X;
+  s.ld = o.ld;
+  s.nvec = o.nvec;
+  s.nvec_pad = o.nvec_pad;
+  s.shifts = o.shifts;
+  s.planes = static_cast<uint16_t*>(o.planes);
+  s.colmax = o.colmax;
+  s.kind = o.contiguous ? (k_pad <= 1024 ? kSideWarp : kSideRow) : k_pad <= kStripMaxK ? kSideStrip : kSideTile;
+  s.blocks2 = 0;
+  switch (s.kind) {
+    case kSideRow: s.blocks1 = (int)o.nvec_pad; break;
+    case kSideWarp: s.blocks1 = (int)(o.nvec_pad / 8); break;
+    case kSideStrip: s.blocks1 = (int)(o.nvec_pad / kColTileJ) * kStripCtas; break;
+    default:
+      s.blocks1 = (int)((o.nvec + 31) / 32 * ((len + 255) / 256));
+      s.blocks2 = (int)(o.nvec_pad / kColTileJ * (k_pad / kColTileH));
+  }
+  return s;
+}
+
+}  // namespace
+
+cudaError_t launch_split_both(const OzTables& t, const SplitOperand& A, const SplitOperand& B, int64_t len,
+                              int64_t k_pad, int32_t* status, cudaStream_t st) {
+  // block counts fit an int
+  if ((A.nvec_pad + B.nvec_pad) / kColTileJ * (k_pad / kColTileH) > INT32_MAX || A.nvec_pad + B.nvec_pad > INT32_MAX / 2)
+    return cudaErrorInvalidValue;
+  const SplitSide a = split_side(A, len, k_pad), b = split_side(B, len, k_pad);
+  switch (pieces_for(t.bits)) {
+    case 4:
+      return t.Q == 16 ? split_both_qt<4, 16>(t, a, b, len, k_pad, status, st)
+                       : split_both_qt<4, 0>(t, a, b, len, k_pad, status, st);
+    case 5: return split_both_qt<5, 0>(t, a, b, len, k_pad, status, st);
+    default: return split_both_qt<7, 0>(t, a, b, len, k_pad, status, st);
+  }
+}
 
 cudaError_t launch_split_rows(const OzTables& t, int64_t nvec, int64_t len, const double* X, int64_t ld,
                               int64_t nvec_pad, int64_t k_pad, int32_t* shifts, void* planes, int bf16,
