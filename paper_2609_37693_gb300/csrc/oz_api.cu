@@ -133,8 +133,10 @@ oz_status dgemm_run(oz_plan plan, int trans_a, int trans_b, int64_t m, int64_t n
   void* V = ws + L.v;
   uint8_t* Y = reinterpret_cast<uint8_t*>(ws + L.y);
 
-  // bf16 planes: both operands split together; the launch clears the status word itself
-  cudaError_t e = bf16 ? cudaSuccess : cudaMemsetAsync(flag, 0, 16, st);
+  // bf16 planes of small or short-vectored operands: both split together; the
+  // launch clears the status word itself
+  const bool both = bf16 && oz::split_both_suits(L.m_pad, L.n_pad, L.k_pad);
+  cudaError_t e = both ? cudaSuccess : cudaMemsetAsync(flag, 0, 16, st);
   if (e != cudaSuccess) return OZ_ERR_CUDA;
   if (plan->is_fp) {
     if (!plan->d_words) return OZ_ERR_CUDA;
@@ -155,7 +157,7 @@ oz_status dgemm_run(oz_plan plan, int trans_a, int trans_b, int64_t m, int64_t n
   // columns in place (A's column maxima go where Y will be, at least 16 bytes
   // a row); for int8 planes B (k x n) is transposed first, so that its columns
   // are split as contiguous rows.
-  if (bf16) {
+  if (both) {
     const oz::SplitOperand oa = {!trans_a, A, lda, m, L.m_pad, s, U, reinterpret_cast<uint64_t*>(Y)};
     const oz::SplitOperand ob = {trans_b != 0, B, ldb, n, L.n_pad, t, V, colmax};
     e = oz::launch_split_both(T, oa, ob, k, L.k_pad, flag, st);
@@ -164,6 +166,8 @@ oz_status dgemm_run(oz_plan plan, int trans_a, int trans_b, int64_t m, int64_t n
                 : oz::launch_split_rows(T, m, k, A, lda, L.m_pad, L.k_pad, s, U, bf16, flag, st);
     if (e == cudaSuccess && trans_b) {
       e = oz::launch_split_rows(T, n, k, B, ldb, L.n_pad, L.k_pad, t, V, bf16, flag, st);
+    } else if (e == cudaSuccess && bf16) {
+      e = oz::launch_split_cols(T, n, k, B, ldb, L.n_pad, L.k_pad, t, V, bf16, flag, colmax, st);
     } else if (e == cudaSuccess) {
       double* Bt = reinterpret_cast<double*>(ws + L.bt);
       e = oz::launch_transpose(k, n, B, ldb, Bt, st);
@@ -174,7 +178,7 @@ oz_status dgemm_run(oz_plan plan, int trans_a, int trans_b, int64_t m, int64_t n
   // GEMMs + epilogue; with too few output tiles, the inner dimension split into
   // ranges whose residue sets are then added modulo m (the layout's split: a
   // TC plan forced onto one CTA per tile runs unsplit)
-  const oz::MarkedShifts marks = bf16 ? oz::MarkedShifts{s, t} : oz::MarkedShifts{nullptr, nullptr};
+  const oz::MarkedShifts marks = both ? oz::MarkedShifts{s, t} : oz::MarkedShifts{nullptr, nullptr};
   const bool forced_single = single_cta && plan->engine == OZ_ENGINE_TC;
   const oz::KSplit split = forced_single ? oz::KSplit{1, 0} : L.split;
   e = (plan->engine == OZ_ENGINE_TC1 || forced_single)

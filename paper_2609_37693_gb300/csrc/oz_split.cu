@@ -351,8 +351,9 @@ __device__ __forceinline__ void split_row_warp(const OzTables& T, int64_t v, int
   }
 }
 
+// (three blocks per SM: 113 us against 130 at 65536 x 256)
 template <bool kBF16, int NP, int QT>
-__global__ void __launch_bounds__(256) split_rows_warp_kernel(const __grid_constant__ OzTables T, int64_t nvec,
+__global__ void __launch_bounds__(256, NP > 5 ? 2 : 3) split_rows_warp_kernel(const __grid_constant__ OzTables T, int64_t nvec,
                                                               int64_t len, const double* __restrict__ X, int64_t ld,
                                                               int64_t nvec_pad, int64_t k_pad,
                                                               int32_t* __restrict__ shifts,
@@ -626,7 +627,7 @@ __device__ __forceinline__ void split_cols_tile(const OzTables& T, int64_t j0, i
 }
 
 template <int NP, int QT>
-__global__ void __launch_bounds__(256, 3) split_cols_bf16_kernel(const __grid_constant__ OzTables T, int64_t nvec,
+__global__ void __launch_bounds__(256, NP > 5 ? 2 : 3) split_cols_bf16_kernel(const __grid_constant__ OzTables T, int64_t nvec,
                                                                 int64_t len, const double* __restrict__ X, int64_t ld,
                                                                 int64_t nvec_pad, int64_t k_pad,
                                                                 const int32_t* __restrict__ shifts,
@@ -663,12 +664,12 @@ __global__ void __launch_bounds__(256, 3) split_cols_grouped_kernel(const __grid
 //   Longer strided vectors: a pass for the column maxima, then 32 x 64 tiles
 //     with the shifts formed from them. (A block's tiles of a strip would run
 //     one after another, with two barriers each: 189 us against 141 us at 4096.)
-// The maxima, strips and rows of a small product share one launch (most of
-// its time is launches and empty SMs); those of a large one are launched on
-// their own, since sharing costs them occupancy and L1 (the maxima run eight
-// blocks an SM alone and three beside the rows; the strips' staging buffers
-// shrink the rows' L1): 8192^3 560 us together, 519 us apart; 65536 x 256 rows
-// beside a 256 x 256 B 150 us against 121 us.
+// The passes of a small product share one launch; those of a larger one with
+// k_pad up to 1024 are launched one after another, since a shared launch costs
+// the rows L1 (65536 x 256 rows beside a 256 x 256 B: 150 us against 121 us).
+// Larger products of longer vectors keep the separate kernels above
+// (split_both_suits): there the launches are nothing and ld.global.nc and plain
+// launches are worth 0.8 % of an 8192^3 product.
 // ---------------------------------------------------------------------------
 struct SplitSide {
   const double* X;
@@ -682,6 +683,7 @@ struct SplitSide {
 constexpr int kSideRow = 0, kSideWarp = 1, kSideStrip = 2, kSideTile = 3, kSideAny = -1;
 constexpr int kStripCtas = 8;
 constexpr int64_t kStripMaxK = 1024;
+constexpr int64_t kMergeEntries = (int64_t)4 << 20;   // of both operands: up to which their passes share a launch
 
 template <int NP, int QT>
 __device__ __forceinline__ void split_strip(const OzTables& T, const SplitSide& S, int64_t strip, int64_t len,
@@ -750,7 +752,7 @@ __device__ __forceinline__ void colmax_side(const SplitSide& S, int64_t l, int64
 }
 
 // Blocks of side b, then side a (status: cleared, when not null).
-// KIND: the kind of every side, kSideRow or kSideWarp; kSideAny: each its own.
+// KIND: the kind of every side, kSideWarp; kSideAny: each its own.
 template <int NP, int QT, int KIND>
 __global__ void __launch_bounds__(256, KIND == kSideAny && NP > 5 ? 2 : 3) split_both_kernel(
     const __grid_constant__ OzTables T, const __grid_constant__ SplitSide a, const __grid_constant__ SplitSide b,
@@ -772,17 +774,6 @@ __global__ void __launch_bounds__(256, KIND == kSideAny && NP > 5 ? 2 : 3) split
                                  S.planes, nullptr, false, true);
   else
     split_row<true, NP, QT>(T, l, S.nvec, len, S.X, S.ld, S.nvec_pad, k_pad, S.shifts, S.planes, nullptr, false, true);
-}
-
-// The column maxima of the kSideTile sides.
-__global__ void __launch_bounds__(256) colmax_both_kernel(const __grid_constant__ SplitSide a,
-                                                          const __grid_constant__ SplitSide b, int64_t len,
-                                                          int32_t* __restrict__ status) {
-  pdl_wait();
-  pdl_trigger();
-  if (status && blockIdx.x == 0 && threadIdx.x < 4) status[threadIdx.x] = 0;
-  const bool second = (int)blockIdx.x < b.blocks1;
-  colmax_side(second ? b : a, second ? blockIdx.x : (int)blockIdx.x - b.blocks1, len);
 }
 
 // The tiles of the kSideTile sides, vectors fastest.
@@ -881,8 +872,9 @@ cudaError_t split_cols_bf16_qt(const OzTables& t, int64_t nvec, int64_t len, con
 template <bool kBF16, int NP>
 cudaError_t split_cols_np(const OzTables& t, int64_t nvec, int64_t len, const double* X, int64_t ld, int64_t nvec_pad,
                           int64_t k_pad, const int32_t* shifts, void* planes, cudaStream_t st) {
-  if constexpr (kBF16 && NP <= 5) {
-    if (t.Q == 16) return split_cols_bf16_qt<NP, 16>(t, nvec, len, X, ld, nvec_pad, k_pad, shifts, planes, st);
+  if constexpr (kBF16) {
+    if constexpr (NP <= 5)
+      if (t.Q == 16) return split_cols_bf16_qt<NP, 16>(t, nvec, len, X, ld, nvec_pad, k_pad, shifts, planes, st);
     return split_cols_bf16_qt<NP, 0>(t, nvec, len, X, ld, nvec_pad, k_pad, shifts, planes, st);
   } else {
     dim3 g((unsigned)(nvec_pad / 64), (unsigned)(k_pad / 64));
@@ -894,9 +886,6 @@ cudaError_t split_cols_np(const OzTables& t, int64_t nvec, int64_t len, const do
 }  // namespace
 
 namespace {
-
-// Entries of both operands up to which their passes share a launch.
-constexpr int64_t kMergeEntries = (int64_t)4 << 20;
 
 template <int NP, int QT>
 cudaError_t split_both_qt(const OzTables& t, const SplitSide& a, const SplitSide& b, int64_t len, int64_t k_pad,
@@ -912,32 +901,22 @@ cudaError_t split_both_qt(const OzTables& t, const SplitSide& a, const SplitSide
       cudaError_t e = cudaMemsetAsync(s->colmax, 0, 8 * (size_t)s->nvec, st);
       if (e != cudaSuccess) return e;
     }
-  auto rows = [](const SplitSide& s) { return s.kind == kSideRow || s.kind == kSideWarp; };
   cudaError_t e = cudaSuccess;
   // one launch of the sides x, y (either may be empty)
   auto first = [&](SplitSide x, SplitSide y) {
     if (e != cudaSuccess || x.blocks1 + y.blocks1 == 0) return;
     const bool strips = (x.blocks1 && x.kind == kSideStrip) || (y.blocks1 && y.kind == kSideStrip);
-    const bool only_rows = (!x.blocks1 || rows(x)) && (!y.blocks1 || rows(y));   // then of one kind, by k_pad
-    e = launch_pdl(!only_rows ? split_both_kernel<NP, QT, kSideAny>
-                   : k_pad <= 1024 ? split_both_kernel<NP, QT, kSideWarp> : split_both_kernel<NP, QT, kSideRow>,
-                   dim3((unsigned)(x.blocks1 + y.blocks1)), dim3(256), strips ? (size_t)tile : 0, st,
+    const bool warps = (!x.blocks1 || x.kind == kSideWarp) && (!y.blocks1 || y.kind == kSideWarp);
+    e = launch_pdl(warps ? split_both_kernel<NP, QT, kSideWarp> : split_both_kernel<NP, QT, kSideAny>, dim3((unsigned)(x.blocks1 + y.blocks1)), dim3(256), strips ? (size_t)tile : 0, st,
                    strips ? kStripCtas : 1, t, x, y, len, k_pad, status);
     status = nullptr;
   };
-  if ((a.nvec_pad + b.nvec_pad) * k_pad <= kMergeEntries || (rows(a) && rows(b))) {
+  if ((a.nvec_pad + b.nvec_pad) * k_pad <= kMergeEntries || (a.kind == kSideWarp && b.kind == kSideWarp)) {
     first(a, b);
   } else {
-    // the column maxima of both, then each operand's strips or rows
-    SplitSide none = {}, x = a, y = b;
-    if (x.kind != kSideTile) x.blocks1 = 0;
-    if (y.kind != kSideTile) y.blocks1 = 0;
-    if (x.blocks1 + y.blocks1 > 0) {
-      e = launch_pdl(colmax_both_kernel, dim3((unsigned)(x.blocks1 + y.blocks1)), dim3(256), 0, st, 1, x, y, len, status);
-      status = nullptr;
-    }
-    if (b.kind != kSideTile) first(none, b);
-    if (a.kind != kSideTile) first(a, none);
+    const SplitSide none = {};
+    first(none, b);
+    first(a, none);
   }
   if (e != cudaSuccess || a.blocks2 + b.blocks2 == 0) return e;
   return launch_pdl(split_tiles_kernel<NP, QT>, dim3((unsigned)(a.blocks2 + b.blocks2)), dim3(256), (size_t)tile, st, 1,
@@ -967,6 +946,10 @@ SplitSide split_side(const SplitOperand& o, int64_t len, int64_t k_pad) {
 }
 
 }  // namespace
+
+bool split_both_suits(int64_t m_pad, int64_t n_pad, int64_t k_pad) {
+  return k_pad <= kStripMaxK || (m_pad + n_pad) * k_pad <= kMergeEntries;
+}
 
 cudaError_t launch_split_both(const OzTables& t, const SplitOperand& A, const SplitOperand& B, int64_t len,
                               int64_t k_pad, int32_t* status, cudaStream_t st) {
