@@ -406,7 +406,7 @@ __device__ __forceinline__ void fold_gemm(uint32_t (&acc16)[NCH * 16], uint32_t 
       __syncwarp();
       if ((threadIdx.x & 31) == 0) {
         if (PAIR) mbar_arrive_cluster(tempty);
-        else mbar_arrive(tempty);
+        else mbar_arrive_relaxed(tempty);
       }
     }
     // the two entries of a word of acc16 go through each packed fp32

@@ -22,8 +22,8 @@
 //   warp 1      allocates all 512 TMEM columns (two 256-column FP32
 //               accumulators) and, from one thread, issues tcgen05.mma
 //               (K = 16) and tcgen05.commit;
-//   warps 2..   E epilogue warps (16 in the one-CTA kernels; 4 or 16 in the
-//               pair kernel, see kPairEpiWarps): drain an accumulator with
+//   warps 2..   E epilogue warps (16; 8 in the pair kernel for products of
+//               several slabs, see kPairEpiWarps): drain an accumulator with
 //               tcgen05.ld while the MMAs fill the other; each slab's sums
 //               are reduced modulo m and written back into the accumulator,
 //               on which the slab after next accumulates; the last two slabs
@@ -234,14 +234,27 @@ __device__ __forceinline__ uint32_t bytes4(const uint32_t* v, uint32_t a8, bool 
                      __byte_perm(__float_as_uint(o1.x), __float_as_uint(o1.y), 0x0040u), 0x5410u);
 }
 
-// One thread's 128 digits of a tile row (one byte each, packed in words) to
+// The digits already in Y that a thread's 16-byte runs will be added to (blocked
+// call): read past L1, and by the callers before the wait for a tile's last
+// slab, so that the reads run under its products. Read run by run between the
+// stores, they held up the drains of the next tile (8192^3 slab 14.2 ms instead
+// of 8.7).
+template <int NW>
+__device__ __forceinline__ void load_old_digits(uint4 (&old)[NW / 4], const uint8_t* dst, int left) {
+  const int chunks = min(NW / 4, (left + 15) >> 4);
+#pragma unroll
+  for (int i = 0; i < NW / 4; ++i)
+    if (i < chunks) old[i] = __ldcg(reinterpret_cast<const uint4*>(dst) + i);
+}
+
+// One thread's 4 NW digits of a tile row (one byte each, packed in words) to
 // Y: whole 16-byte runs up to `left` (the columns of the row from here to n)
 // rounded up to 16 when the row pitch is a multiple of 16 (bytes past n are
-// never read), byte stores otherwise. acc: add into the digits in Y modulo m.
+// never read), byte stores otherwise. acc: add into the digits in Y modulo m
+// (the runs' from old).
 template <int NW>
 __device__ __forceinline__ void store_digits(uint8_t* dst, const uint32_t* w, int left, bool runs, int acc,
-                                             uint32_t m) {
-  static_assert(NW == 32 || NW == 16, "128 or 64 digits");
+                                             uint32_t m, const uint4* old) {
   if (runs) {
     const int chunks = min(NW / 4, (left + 15) >> 4);
     const uint32_t mm = m * 0x01010101u;
@@ -250,11 +263,10 @@ __device__ __forceinline__ void store_digits(uint8_t* dst, const uint32_t* w, in
       if (i < chunks) {
         uint4 o = make_uint4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]);
         if (acc) {
-          const uint4 old = reinterpret_cast<const uint4*>(dst)[i];
-          o.x = addmod_bytes(o.x, old.x, mm);
-          o.y = addmod_bytes(o.y, old.y, mm);
-          o.z = addmod_bytes(o.z, old.z, mm);
-          o.w = addmod_bytes(o.w, old.w, mm);
+          o.x = addmod_bytes(o.x, old[i].x, mm);
+          o.y = addmod_bytes(o.y, old[i].y, mm);
+          o.z = addmod_bytes(o.z, old[i].z, mm);
+          o.w = addmod_bytes(o.w, old[i].w, mm);
         }
         reinterpret_cast<uint4*>(dst)[i] = o;
       }
@@ -277,8 +289,7 @@ __device__ __forceinline__ void store_digits(uint8_t* dst, const uint32_t* w, in
 
 // The drain of a unit that is one slab (a kernel launched for K of at most
 // 1024 terms, unsplit): every chunk of this warp's columns is loaded first and
-// the accumulator released at once (one arrival per warp: each thread's
-// release-ordered arrival cost a memory barrier per unit), so that the
+// the accumulator released at once (one arrival per warp), so that the
 // products of the unit after next start while this warp forms the digits
 // (W mod m reduced exactly, then the CRT digit, or W mod m when raw), one byte
 // per entry in acc8.
@@ -299,7 +310,6 @@ __device__ __forceinline__ void drain_one_slab(uint32_t taddr0, uint32_t (&acc8)
 
 struct Params {
   int m, n, tiles_m, tiles_n, num_tiles, kblocks, m_pad, n_pad, raw;
-  int acc;           // add into the digits already in Y, modulo m (blocked call)
   uint8_t* Y;
   int64_t ldy;       // row pitch of Y
   int32_t* status;
@@ -330,8 +340,10 @@ __device__ __forceinline__ Unit unit_of(const Params& p, int u) {
   return w;
 }
 
-// ONE: every unit is one slab (K <= 1024, unsplit); see drain_one_slab.
-template <bool ONE>
+// ONE: every unit is one slab (K <= 1024, unsplit); see drain_one_slab. ACC: the
+// digits are added into those in Y (a kernel of its own: the old digits' registers
+// cost the 65536 x 256 x 256 GEMM 18 %).
+template <bool ONE, bool ACC>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const __grid_constant__ OzTables T, const Params p) {
@@ -359,7 +371,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(tfull_bar(b), 1);
-      mbar_init(tempty_bar(b), ONE ? kEpiWarps : kEpiWarps * 32);   // one-slab: one arrival per warp
+      mbar_init(tempty_bar(b), kEpiWarps);      // one arrival per warp
     }
     mbar_init(drain_bar, 1);
     *abort_flag = 0;
@@ -464,11 +476,19 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       const Coord c = u.c;
       const int nslabs = u.nslabs;
       const EpiConst k = epi_const((float)T.m[c.q], T.invm[c.q], p.raw ? 1.0f : (float)T.inv[c.q]);
+      const int row = c.tm * BM + quarter * 32 + lane;
+      const int col0 = c.tn * BN + cbase;
+      const bool in = row < p.m && col0 < p.n;
+      const bool runs = (p.ldy & 15) == 0 && (reinterpret_cast<uintptr_t>(p.Y) & 15) == 0;
+      uint8_t* const dst = p.Y + (size_t)u.ks * p.ysplit + (size_t)c.q * p.m * p.ldy + (size_t)row * p.ldy + col0;
+      uint4 old[ACC ? CPW1 / 16 : 1];
       uint32_t acc8[CPW1 / 4];
 #pragma unroll
       for (int i = 0; i < CPW1 / 4; ++i) acc8[i] = 0x80808080u;
       for (int sl = 0; sl < nslabs; ++sl, ++g) {
         const uint32_t b = g & 1u, use = g >> 1;
+        if constexpr (ACC)
+          if (sl + 1 == nslabs && in && runs) load_old_digits<CPW1 / 4>(old, dst, p.n - col0);
         if (!mbar_wait(tfull_bar(b), use & 1u, abort_flag, p.status)) { ok = false; break; }
         tc_fence_after();
         if constexpr (ONE) {
@@ -476,7 +496,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           drain_one_slab<CPW1 / 32>(tmem_base + lane_addr + b * BN + cbase, acc8, k,
                                     [&] {
                                       __syncwarp();
-                                      if (lane == 0) mbar_arrive(tb);
+                                      if (lane == 0) mbar_arrive_relaxed(tb);
                                     });
           continue;
         }
@@ -498,17 +518,12 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         }
         if (write_back) tmem_st_wait();
         tc_fence_before();
-        mbar_arrive(tempty_bar(b));
+        __syncwarp();
+        if (lane == 0) mbar_arrive_relaxed(tempty_bar(b));
       }
       if (!ok) break;
       // ---- tile done: acc8 holds the digits (or W mod m), one byte per entry ----
-      const int row = c.tm * BM + quarter * 32 + lane;
-      const int col0 = c.tn * BN + cbase;
-      if (row < p.m && col0 < p.n) {
-        uint8_t* dst = p.Y + (size_t)u.ks * p.ysplit + (size_t)c.q * p.m * p.ldy + (size_t)row * p.ldy + col0;
-        store_digits<CPW1 / 4>(dst, acc8, p.n - col0, (p.ldy & 15) == 0 && (reinterpret_cast<uintptr_t>(p.Y) & 15) == 0,
-                               p.acc, T.m[c.q]);
-      }
+      if (in) store_digits<CPW1 / 4>(dst, acc8, p.n - col0, runs, ACC, T.m[c.q], old);
     }
   }
 
@@ -540,13 +555,13 @@ constexpr int P_SMEM_BYTES = P_STAGES * P_STAGE_BYTES + kBarBytes + 1024;
 // full and empty barriers per stage, two tfull, two tempty, one drain: all below kHolderOff
 static_assert((2 * P_STAGES + 5) * 8 <= kHolderOff, "pair kernel barriers overlap the TMEM address");
 static_assert((2 * STAGES + 5) * 8 <= kHolderOff, "barriers overlap the TMEM address");
-// Epilogue warps of the pair kernel: sixteen when every unit is one slab
-// (the epilogue then bounds the kernel) and for grouped products; four for a
-// product of several slabs, where fewer warps beside the MMA-issuing thread
-// leave it more issue slots: with the packed epilogue arithmetic one warp
-// drains its 256 columns of a slab well within the slab's products.
+// Epilogue warps of the pair kernel: sixteen when every unit is one slab (the
+// epilogue then bounds the kernel) and for grouped products; eight for one
+// product of several slabs: 8192^3 products 11.3 ms under the power cap against
+// 11.5 with four or sixteen, 4096^3 1.57 ms with any, 2048^3 GEMMs 170 us
+// against 172 and 169.
 constexpr int kPairEpiWarps = 16;
-constexpr int kPairEpiWarpsMulti = 4;
+constexpr int kPairEpiWarpsMulti = 8;
 
 // What a CTA pair needs to know about one unit of work: the tensor maps and
 // first plane rows of its 256 x 256 tile, its k-block range, its modulus and
@@ -560,7 +575,7 @@ struct PairUnit {
   uint8_t* Y;               // digit plane of this unit (row pitch ldy, m rows, n columns)
   int64_t ldy;
   int m, n, row0, col0;     // the output's size and the tile's first row and column
-  int acc, raw;
+  int raw;
 };
 
 // One product (oz_dgemm): units are (split, modulus, tile), as unit_of orders them.
@@ -592,7 +607,6 @@ struct PairSingle {
     w.n = p.n;
     w.row0 = u.c.tm * 2 * P_BM;
     w.col0 = u.c.tn * 2 * P_BN;
-    w.acc = p.acc;
     w.raw = p.raw;
     return w;
   }
@@ -634,20 +648,18 @@ struct PairGrouped {
     w.n = (int)P.n;
     w.row0 = c.tm * 2 * P_BM;
     w.col0 = c.tn * 2 * P_BN;
-    w.acc = 0;
     w.raw = 0;
     return w;
   }
 };
 
-// EW epilogue warps (4, 8 or 16): every warp drains the 32 TMEM lanes of its
-// quarter (warp index mod 4), over CPW = 256 / (EW / 4) columns.
+// EW epilogue warps: every warp drains the 32 TMEM lanes of its quarter (warp
+// index mod 4), over CPW = 256 / (EW / 4) columns.
 // S: the unit scheduler (PairSingle or PairGrouped).
-template <int EW, typename S, bool ONE>
+template <int EW, typename S, bool ONE, bool ACC>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__((2 + EW) * 32, 1)
 gemm_tc_pair_kernel(const __grid_constant__ S sched, const __grid_constant__ OzTables T) {
   constexpr int CPW = 1024 / EW;            // columns per epilogue warp
-  static_assert(EW == 4 || EW == 8 || EW == 16, "4, 8 or 16 epilogue warps");
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw_base = smem_u32(smem_raw);
   const uint32_t base = (raw_base + 1023u) & ~1023u;
@@ -674,7 +686,7 @@ gemm_tc_pair_kernel(const __grid_constant__ S sched, const __grid_constant__ OzT
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(tfull_bar(b), 1);
-      mbar_init(tempty_bar(b), ONE ? 2 * EW : 2 * EW * 32);        // one-slab: one arrival per warp
+      mbar_init(tempty_bar(b), 2 * EW);        // one arrival per warp
     }
     mbar_init(drain_bar, 1);
     *abort_flag = 0;
@@ -788,11 +800,19 @@ gemm_tc_pair_kernel(const __grid_constant__ S sched, const __grid_constant__ OzT
       const PairUnit u = sched.unit(t, pi);
       const int nslabs = u.nslabs;
       const EpiConst k = epi_const((float)T.m[u.q], T.invm[u.q], u.raw ? 1.0f : (float)T.inv[u.q]);
+      const int row = u.row0 + (int)rank * P_BM + quarter * 32 + lane;
+      const int col0 = u.col0 + cbase;
+      const bool in = row < u.m && col0 < u.n;
+      const bool runs = (u.ldy & 15) == 0 && (reinterpret_cast<uintptr_t>(u.Y) & 15) == 0;
+      uint8_t* const dst = u.Y + (size_t)row * u.ldy + col0;
+      uint4 old[ACC ? CPW / 16 : 1];
       uint32_t acc8[CPW / 4];                // residue + 128 of the chain of slab nsl - 2, one byte per column
 #pragma unroll
       for (int i = 0; i < CPW / 4; ++i) acc8[i] = 0x80808080u;
       for (int sl = 0; sl < nslabs; ++sl, ++g) {
         const uint32_t b = g & 1u, use = g >> 1;
+        if constexpr (ACC)
+          if (sl + 1 == nslabs && in && runs) load_old_digits<CPW / 4>(old, dst, u.n - col0);
         if (!mbar_wait(tfull_bar(b), use & 1u, abort_flag, status)) { ok = false; break; }
         tc_fence_after();
         if constexpr (ONE) {
@@ -822,20 +842,12 @@ gemm_tc_pair_kernel(const __grid_constant__ S sched, const __grid_constant__ OzT
         }
         if (write_back) tmem_st_wait();
         tc_fence_before();
-        mbar_arrive_cluster(mapa(tempty_bar(b), 0));
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(mapa(tempty_bar(b), 0));
       }
       if (!ok) break;
       // ---- tile done: acc8 holds the digits (or W mod m), one byte per entry ----
-      const int row = u.row0 + (int)rank * P_BM + quarter * 32 + lane;
-      const bool runs = (u.ldy & 15) == 0 && (reinterpret_cast<uintptr_t>(u.Y) & 15) == 0;
-#pragma unroll
-      for (int part = 0; part < (CPW + 127) / 128; ++part) {
-        const int col0 = u.col0 + cbase + part * 128;
-        if (row < u.m && col0 < u.n) {
-          uint8_t* dst = u.Y + (size_t)row * u.ldy + col0;
-          store_digits<(CPW < 128 ? CPW : 128) / 4>(dst, acc8 + part * 32, u.n - col0, runs, u.acc, T.m[u.q]);
-        }
-      }
+      if (in) store_digits<CPW / 4>(dst, acc8, u.n - col0, runs, ACC, T.m[u.q], old);
     }
   }
 
@@ -889,7 +901,7 @@ gemm_tc_grouped_kernel(const __grid_constant__ OzTables T, const OzGroupProblem*
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(tfull_bar(b), 1);
-      mbar_init(tempty_bar(b), ONE ? kEpiWarps : kEpiWarps * 32);   // one-slab: one arrival per warp
+      mbar_init(tempty_bar(b), kEpiWarps);      // one arrival per warp
     }
     mbar_init(drain_bar, 1);
     *abort_flag = 0;
@@ -1004,7 +1016,7 @@ gemm_tc_grouped_kernel(const __grid_constant__ OzTables T, const OzGroupProblem*
           drain_one_slab<CPW1 / 32>(tmem_base + lane_addr + b * BN + cbase, acc8, k,
                                     [&] {
                                       __syncwarp();
-                                      if (lane == 0) mbar_arrive(tb);
+                                      if (lane == 0) mbar_arrive_relaxed(tb);
                                     });
           continue;
         }
@@ -1026,7 +1038,8 @@ gemm_tc_grouped_kernel(const __grid_constant__ OzTables T, const OzGroupProblem*
         }
         if (write_back) tmem_st_wait();
         tc_fence_before();
-        mbar_arrive(tempty_bar(b));
+        __syncwarp();
+        if (lane == 0) mbar_arrive_relaxed(tempty_bar(b));
       }
       if (!ok) break;
       const int row = c.tm * BM + quarter * 32 + lane;
@@ -1034,7 +1047,7 @@ gemm_tc_grouped_kernel(const __grid_constant__ OzTables T, const OzGroupProblem*
       if (row < P.m && col0 < P.n) {
         uint8_t* dst = P.Y + (size_t)c.q * P.m * P.ldy + (size_t)row * P.ldy + col0;
         store_digits<CPW1 / 4>(dst, acc8, P.n - col0, (P.ldy & 15) == 0 && (reinterpret_cast<uintptr_t>(P.Y) & 15) == 0,
-                               0, T.m[c.q]);
+                               0, T.m[c.q], nullptr);
       }
     }
   }
@@ -1129,8 +1142,11 @@ cudaError_t launch_gemm_tc(const OzTables& t, int64_t m, int64_t n, int64_t m_pa
   // every unit one slab (K <= 1024, unsplit): the kernel whose epilogue
   // releases each accumulator before forming its digits
   const bool one = k_pad <= (int64_t)kSlabBlocks * BK && split.nsplit <= 1;
-  auto kernel = one ? gemm_tc_pair_kernel<kPairEpiWarps, PairSingle, true>
-                    : gemm_tc_pair_kernel<kPairEpiWarpsMulti, PairSingle, false>;
+  auto kernel = raw & kEpiAccumulate
+                    ? (one ? gemm_tc_pair_kernel<kPairEpiWarps, PairSingle, true, true>
+                           : gemm_tc_pair_kernel<kPairEpiWarpsMulti, PairSingle, false, true>)
+                    : (one ? gemm_tc_pair_kernel<kPairEpiWarps, PairSingle, true, false>
+                           : gemm_tc_pair_kernel<kPairEpiWarpsMulti, PairSingle, false, false>);
   const int epi_warps = one ? kPairEpiWarps : kPairEpiWarpsMulti;
   e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
   if (e != cudaSuccess) return e;
@@ -1147,7 +1163,6 @@ cudaError_t launch_gemm_tc(const OzTables& t, int64_t m, int64_t n, int64_t m_pa
   p.m_pad = (int)m_pad;
   p.n_pad = (int)n_pad;
   p.raw = raw & kEpiRaw;
-  p.acc = (raw & kEpiAccumulate) != 0;
   p.Y = Y;
   p.ldy = ldy;
   p.status = status;
@@ -1181,8 +1196,8 @@ cudaError_t launch_gemm_tc_grouped(const OzTables& t, const OzGroupProblem* prob
     e = cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (e != cudaSuccess) return e;
     const int smem_bytes = smem_optin > P_SMEM_BYTES ? smem_optin : P_SMEM_BYTES;
-    auto kernel = one_slab ? gemm_tc_pair_kernel<kPairEpiWarps, PairGrouped, true>
-                           : gemm_tc_pair_kernel<kPairEpiWarps, PairGrouped, false>;
+    auto kernel = one_slab ? gemm_tc_pair_kernel<kPairEpiWarps, PairGrouped, true, false>
+                           : gemm_tc_pair_kernel<kPairEpiWarps, PairGrouped, false, false>;
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
     if (e != cudaSuccess) return e;
     PairGrouped sched;
@@ -1225,7 +1240,8 @@ cudaError_t launch_gemm_tc_single(const OzTables& t, int64_t m, int64_t n, int64
   e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
   const bool one = k_pad <= (int64_t)kSlabBlocks * BK && split.nsplit <= 1;
-  auto kernel = one ? gemm_tc_kernel<true> : gemm_tc_kernel<false>;
+  auto kernel = raw & kEpiAccumulate ? (one ? gemm_tc_kernel<true, true> : gemm_tc_kernel<false, true>)
+                                     : (one ? gemm_tc_kernel<true, false> : gemm_tc_kernel<false, false>);
   e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
   if (e != cudaSuccess) return e;
   Params p;
@@ -1238,7 +1254,6 @@ cudaError_t launch_gemm_tc_single(const OzTables& t, int64_t m, int64_t n, int64
   p.m_pad = (int)m_pad;
   p.n_pad = (int)n_pad;
   p.raw = raw & kEpiRaw;
-  p.acc = (raw & kEpiAccumulate) != 0;
   p.Y = Y;
   p.ldy = ldy;
   p.status = status;

@@ -33,8 +33,12 @@ static __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUte
       "l"(map), "r"(bar_cluster), "r"(x), "r"(y)
       : "memory");
 }
+// Relaxed: what an epilogue hands over with this arrival is tensor memory,
+// ordered by tcgen05.wait and tcgen05.fence::before_thread_sync. A release at
+// cluster scope is a memory barrier that also waits for the warp's digit stores
+// to global memory (the top stall of the 65536 x 256 x 256 GEMM).
 static __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar_cluster) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster) : "memory");
+  asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster) : "memory");
 }
 static __device__ __forceinline__ void tmem_alloc_pair(uint32_t dst_smem, uint32_t ncols) {
   asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst_smem), "r"(ncols)
