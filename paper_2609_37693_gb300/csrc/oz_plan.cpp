@@ -128,13 +128,15 @@ namespace oz {
 // unset (rg_nt = rg_np2 = rg_nq4 = 0) unless every bound the kernel relies on
 // holds: digits and moduli below 256 (dp2a takes bytes), weights below 2^16,
 // the sum of the groups' largest t_g below 2^32 (each 64-bit limb
-// accumulator then stays below 2^64), N_g below 2^128, the CRT sum below
-// 15 P (its quotient fits the kernel's table of 16 multiples of P), and
-// 3P / 2 below 2^127 (the two's-complement candidate X).
+// accumulator then stays below 2^64), and with L = 4 limbs up to Q = 16 and 5
+// above: N_g below 2^(32 L), the CRT sum below 15 P (23 P; its quotient fits the
+// kernel's table of 16 or 24 multiples of P), and 3P / 2 below 2^(32 L - 1)
+// (the two's-complement candidate X).
 void fill_group_tables(OzTables* tp, const uint32_t* moduli, int Q, const Big& P) {
   OzTables& t = *tp;
   t.rg_nt = t.rg_np2 = t.rg_nq4 = 0;
-  if (Q < 2 || Q > 16 || P.bitlen() > 125) return;
+  const int limbs = Q <= 16 ? 4 : 5;
+  if (Q < 2 || Q > 20 || P.bitlen() > 32 * limbs - 3) return;
   for (int q = 0; q < Q; ++q)
     if (moduli[q] >= 256) return;
   int nt = Q / 3, np2 = 0, nq4 = 0;
@@ -186,12 +188,12 @@ void fill_group_tables(OzTables* tp, const uint32_t* moduli, int Q, const Big& P
       N.divmod(moduli[q + i], &N2);
       N = N2;
     }
-    if (N.bitlen() > 128) return;
-    for (int l = 0; l < 4; ++l) t.rg_N[g][l] = N.w[l];
+    if (N.bitlen() > 32 * limbs) return;
+    for (int l = 0; l < 5; ++l) t.rg_N[g][l] = N.w[l];
     t.rg_invM[g] = (float)(1.0 / (double)Mg);
     q += size;
   }
-  if (q != Q || tsum >= 4294967296.0 || ksum > 15.0) return;
+  if (q != Q || tsum >= 4294967296.0 || ksum > (limbs == 4 ? 15.0 : 23.0)) return;
   t.rg_nt = nt;
   t.rg_np2 = np2;
   t.rg_nq4 = nq4;

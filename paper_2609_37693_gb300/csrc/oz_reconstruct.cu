@@ -484,70 +484,103 @@ __device__ __forceinline__ uint32_t group_t(int g, const uint32_t* w, int e, uin
   return wab * m2b + wcd * m2a;                    // < 2 M_4 < 2^32
 }
 
-// The CRT sum of entry e of the digit words w[0..Q-1]: S modulo 2^128 as
-// 32-bit limbs s[0..3], and f = sum_g fl(t_g) fl(1 / M_g), an estimate of
-// S / P. Per limb l, a_l = sum_g t_g n_{g,l} in 64 bits (below 2^64: the sum
-// of the largest t_g is below 2^32); only the low 32 bits of a_3 reach S.
-template <int NT, int NP2, int NQ4>
-__device__ __forceinline__ void crt_groups(const OzTables& T, const uint32_t* w, int e, uint32_t (&s)[4], float& f) {
-  uint64_t a0 = 0, a1 = 0, a2 = 0;
-  uint32_t a3 = 0;
+// 32-bit limbs of the CRT sum of Q moduli in groups: P < 2^125 (Q <= 16) or
+// P < 2^157 (Q <= 20).
+constexpr int rg_limbs(int Q) { return Q <= 16 ? 4 : 5; }
+// multiples of P in the kernels' tables, more than the sum can reach
+constexpr int rg_multiples(int Q) { return Q <= 16 ? 16 : 24; }
+
+// The CRT sum of entry e of the digit words w[0..Q-1]: S modulo 2^(32 L) as
+// 32-bit limbs, and f = sum_g fl(t_g) fl(1 / M_g), an estimate of S / P. Per
+// limb l, a_l = sum_g t_g n_{g,l} in 64 bits (below 2^64: the sum of the largest
+// t_g is below 2^32); only the low 32 bits of the top one reach S.
+template <int NT, int NP2, int NQ4, int L>
+__device__ __forceinline__ void crt_groups(const OzTables& T, const uint32_t* w, int e, uint32_t (&s)[L], float& f) {
+  static_assert(L == 4 || L == 5, "four or five limbs");
+  uint64_t a[L - 1] = {};
+  uint32_t top = 0;
   f = 0.0f;
 #pragma unroll
   for (int g = 0; g < NT + NP2 + NQ4; ++g) {
     const bool quad = g >= NT + NP2;
     const uint32_t tg = group_t<NT, NP2, NQ4>(g, w, e, T.rg_w0[g], T.rg_w1[g], quad ? T.rg_m2a[g] : 0u,
                                               quad ? T.rg_m2b[g] : 0u);
-    a0 += (uint64_t)tg * T.rg_N[g][0];
-    a1 += (uint64_t)tg * T.rg_N[g][1];
-    a2 += (uint64_t)tg * T.rg_N[g][2];
-    a3 += tg * T.rg_N[g][3];
+#pragma unroll
+    for (int l = 0; l < L - 1; ++l) a[l] += (uint64_t)tg * T.rg_N[g][l];
+    top += tg * T.rg_N[g][L - 1];
     f = fmaf(__uint2float_rn(tg), T.rg_invM[g], f);
   }
-  // S = a0 + a1 2^32 + a2 2^64 + a3 2^96 modulo 2^128
-  s[0] = (uint32_t)a0;
-  asm("add.cc.u32 %0, %3, %4;\n\taddc.cc.u32 %1, %5, %6;\n\taddc.u32 %2, %7, %8;"
-      : "=r"(s[1]), "=r"(s[2]), "=r"(s[3])
-      : "r"((uint32_t)(a0 >> 32)), "r"((uint32_t)a1), "r"((uint32_t)(a1 >> 32)), "r"((uint32_t)a2),
-        "r"((uint32_t)(a2 >> 32)), "r"(a3));
+  // S = sum_l a_l 2^(32 l) + top 2^(32 (L - 1))
+  s[0] = (uint32_t)a[0];
+  if constexpr (L == 4)
+    asm("add.cc.u32 %0, %3, %4;\n\taddc.cc.u32 %1, %5, %6;\n\taddc.u32 %2, %7, %8;"
+        : "=r"(s[1]), "=r"(s[2]), "=r"(s[3])
+        : "r"((uint32_t)(a[0] >> 32)), "r"((uint32_t)a[1]), "r"((uint32_t)(a[1] >> 32)), "r"((uint32_t)a[2]),
+          "r"((uint32_t)(a[2] >> 32)), "r"(top));
+  else
+    asm("add.cc.u32 %0, %4, %5;\n\taddc.cc.u32 %1, %6, %7;\n\taddc.cc.u32 %2, %8, %9;\n\taddc.u32 %3, %10, %11;"
+        : "=r"(s[1]), "=r"(s[2]), "=r"(s[3]), "=r"(s[4])
+        : "r"((uint32_t)(a[0] >> 32)), "r"((uint32_t)a[1]), "r"((uint32_t)(a[1] >> 32)), "r"((uint32_t)a[2]),
+          "r"((uint32_t)(a[2] >> 32)), "r"((uint32_t)a[L - 2]), "r"((uint32_t)(a[L - 2] >> 32)), "r"(top));
 }
 
-// x -= y over four 32-bit limbs (modulo 2^128)
-__device__ __forceinline__ void sub128(uint32_t (&x)[4], const uint32_t (&y)[4]) {
-  asm("sub.cc.u32 %0, %0, %4;\n\tsubc.cc.u32 %1, %1, %5;\n\tsubc.cc.u32 %2, %2, %6;\n\tsubc.u32 %3, %3, %7;"
-      : "+r"(x[0]), "+r"(x[1]), "+r"(x[2]), "+r"(x[3])
-      : "r"(y[0]), "r"(y[1]), "r"(y[2]), "r"(y[3]));
+// x -= y over L 32-bit limbs (modulo 2^(32 L))
+template <int L>
+__device__ __forceinline__ void sub_limbs(uint32_t (&x)[L], const uint32_t (&y)[L]) {
+  if constexpr (L == 4)
+    asm("sub.cc.u32 %0, %0, %4;\n\tsubc.cc.u32 %1, %1, %5;\n\tsubc.cc.u32 %2, %2, %6;\n\tsubc.u32 %3, %3, %7;"
+        : "+r"(x[0]), "+r"(x[1]), "+r"(x[2]), "+r"(x[3])
+        : "r"(y[0]), "r"(y[1]), "r"(y[2]), "r"(y[3]));
+  else
+    asm("sub.cc.u32 %0, %0, %5;\n\tsubc.cc.u32 %1, %1, %6;\n\tsubc.cc.u32 %2, %2, %7;\n\tsubc.cc.u32 %3, %3, %8;\n\t"
+        "subc.u32 %4, %4, %9;"
+        : "+r"(x[0]), "+r"(x[1]), "+r"(x[2]), "+r"(x[3]), "+r"(x[4])
+        : "r"(y[0]), "r"(y[1]), "r"(y[2]), "r"(y[3]), "r"(y[4]));
 }
 
-__device__ __forceinline__ u128 to_u128(const uint32_t (&x)[4]) {
-  return ((u128)(((uint64_t)x[3] << 32) | x[2]) << 64) | (((uint64_t)x[1] << 32) | x[0]);
+// q P from the kernel's table of multiples (L words each, 16-byte rows)
+template <int L>
+__device__ __forceinline__ void multiple_of_P(const uint4* kP, int q, uint32_t (&y)[L]) {
+  const uint4 v = kP[L == 4 ? q : 2 * q];
+  y[0] = v.x, y[1] = v.y, y[2] = v.z, y[3] = v.w;
+  if constexpr (L == 5) y[4] = kP[2 * q + 1].x;
 }
 
-// fl(X 2^ex) for X = S - qP, q the quotient estimate; kP[q] = q P (shared),
-// in the usual case: the estimate clear of a tie, 2^96 <= |X| and a normal
-// result. It runs in 32-bit limbs: the magnitude by a sign mask, the leading
-// bit by clz of the top limb, 64 bits below it by funnel shifts, one
-// round-to-nearest-even increment. Returns false (out unset) otherwise.
-__device__ __forceinline__ bool round_groups_fast(const uint4* kP, const uint32_t (&s)[4], float f, int ex,
+// fl(X 2^ex) for X = S - qP, q the quotient estimate, in the usual case: the
+// estimate clear of a tie, |X| >= 2^96 and a normal result. It runs in 32-bit
+// limbs: the magnitude by a sign mask, the leading bit by clz of the top limb
+// that is not zero (five limbs: the fifth or fourth), 64 bits below it by funnel
+// shifts, one round-to-nearest-even increment. Returns false (out unset)
+// otherwise.
+template <int L>
+__device__ __forceinline__ bool round_groups_fast(const uint4* kP, int kmax, const uint32_t (&s)[L], float f, int ex,
                                                   uint64_t& out) {
   const float kf = rintf(f);
-  const int k = min((int)kf, 15);
-  const uint4 kp = kP[k];
-  uint32_t x[4] = {s[0], s[1], s[2], s[3]};
-  const uint32_t kq[4] = {kp.x, kp.y, kp.z, kp.w};
-  sub128(x, kq);
+  uint32_t m[L], y[L];
+  multiple_of_P<L>(kP, min((int)kf, kmax), y);
+#pragma unroll
+  for (int l = 0; l < L; ++l) m[l] = s[l];
+  sub_limbs<L>(m, y);
   // magnitude: (x ^ mask) - mask
-  const uint32_t mask = (uint32_t)((int32_t)x[3] >> 31);
-  uint32_t m[4] = {x[0] ^ mask, x[1] ^ mask, x[2] ^ mask, x[3] ^ mask};
-  const uint32_t mk[4] = {mask, mask, mask, mask};
-  sub128(m, mk);
+  const uint32_t mask = (uint32_t)((int32_t)m[L - 1] >> 31);
+#pragma unroll
+  for (int l = 0; l < L; ++l) m[l] ^= mask, y[l] = mask;
+  sub_limbs<L>(m, y);
+  uint32_t low = 0;                                        // bits below the four limbs rounded
+  int top = 127;
+  if constexpr (L == 5) {
+    if (m[4] != 0) {
+      low = m[0], m[0] = m[1], m[1] = m[2], m[2] = m[3], m[3] = m[4];
+      top = 159;
+    }
+  }
   const int lz = __clz((int)m[3]);
-  const int E = 127 - lz + ex;                             // exponent of the leading bit
+  const int E = top - lz + ex;                             // exponent of the leading bit
   if (fabsf(f - kf) > 0.499f || m[3] == 0 || (unsigned)(E + 1022) > 2045u) return false;
   // 64 bits from the leading one down (h1:h0), and whether any bit below is set
   const uint32_t h1 = __funnelshift_l(m[2], m[3], lz);
   const uint32_t h0 = __funnelshift_l(m[1], m[2], lz);
-  const uint32_t r = __funnelshift_l(m[0], m[1], lz) | (m[0] << lz);
+  const uint32_t r = __funnelshift_l(m[0], m[1], lz) | (m[0] << lz) | low;
   const uint64_t mant = (((uint64_t)h1 << 32) | h0) >> 11;  // 53 bits, leading one at bit 52
   const uint32_t half = (h0 >> 10) & 1u;
   const uint32_t sticky = ((h0 & 0x3ffu) | r) != 0u;
@@ -559,38 +592,59 @@ __device__ __forceinline__ bool round_groups_fast(const uint4* kP, const uint32_
 }
 
 // Every other case, recomputed from the digits (wsm[q * QS], this thread's
-// shared-memory slots): the CRT sum S exactly in 128 bits (S < 15 P < 2^128),
+// shared-memory slots): the CRT sum S exactly (S < kmax P < 2^(32 L)),
 // X = S - qP corrected exactly into [-P/2, P/2), and the general rounding.
 template <int NT, int NP2, int NQ4, int QS>
 __device__ __noinline__ uint64_t round_groups_slow(const OzTables& T, const uint4* kP, const uint32_t* wsm, int e,
                                                    int ex) {
-  constexpr int Q = 3 * NT + 2 * NP2 + 4 * NQ4;
+  constexpr int Q = 3 * NT + 2 * NP2 + 4 * NQ4, L = rg_limbs(Q);
   uint32_t w[Q];
 #pragma unroll
   for (int q = 0; q < Q; ++q) w[q] = wsm[q * QS];
-  uint32_t s[4];
+  uint32_t s[L], y[L];
   float f;
-  crt_groups<NT, NP2, NQ4>(T, w, e, s, f);
-  const int k = min((int)rintf(f), 15);
-  const uint4 kp = kP[k];
-  const uint32_t kq[4] = {kp.x, kp.y, kp.z, kp.w};
-  sub128(s, kq);
-  __int128 X = (__int128)to_u128(s);
-  const uint4 p = kP[1];
-  const u128 P = ((u128)(((uint64_t)p.w << 32) | p.z) << 64) | (((uint64_t)p.y << 32) | p.x);
-  if (2 * X >= (__int128)P) X -= (__int128)P;
-  else if (2 * X < -(__int128)P) X += (__int128)P;
-  const uint32_t neg = X < 0;
-  const u128 mag = neg ? (u128)(-X) : (u128)X;
-  return round128(mag, neg, ex);
+  crt_groups<NT, NP2, NQ4, L>(T, w, e, s, f);
+  multiple_of_P<L>(kP, min((int)rintf(f), rg_multiples(Q) - 1), y);
+  sub_limbs<L>(s, y);
+  Limbs<L> X;
+#pragma unroll
+  for (int l = 0; l < L; ++l) X.w[l] = s[l];
+  if (twice_ge_P(X, T.P)) sub_mul_P(X, 1u, T.P);
+  else if (twice_lt_minus_P(X, T.P)) add_P(X, T.P);
+  const uint32_t neg = X.w[L - 1] >> 31;
+  if (neg) {
+    uint64_t c = 1;
+#pragma unroll
+    for (int l = 0; l < L; ++l) {
+      const uint64_t v = (uint64_t)(~X.w[l]) + c;
+      X.w[l] = (uint32_t)v;
+      c = v >> 32;
+    }
+  }
+  return round_to_binary64(X, neg, ex);
 }
 
-// kP[q] = q P for q = 0..15, as four 32-bit limbs (threads 0..15 of the block)
-__device__ __forceinline__ void fill_kP(const OzTables& T, uint4* kP) {
-  if (threadIdx.x < 16) {
-    const u128 P = ((u128)(((uint64_t)T.P[3] << 32) | T.P[2]) << 64) | (((uint64_t)T.P[1] << 32) | T.P[0]);
-    const u128 v = P * (u128)threadIdx.x;
-    kP[threadIdx.x] = make_uint4((uint32_t)v, (uint32_t)(v >> 32), (uint32_t)(v >> 64), (uint32_t)(v >> 96));
+// The table of multiples q P, q < rg_multiples(Q): one uint4 each (four limbs)
+// or two (five).
+template <int Q>
+struct MultiplesOfP {
+  uint4 v[rg_multiples(Q) * (rg_limbs(Q) == 4 ? 1 : 2)];
+};
+template <int Q>
+__device__ __forceinline__ void fill_kP(const OzTables& T, MultiplesOfP<Q>& kP) {
+  constexpr int L = rg_limbs(Q);
+  if (threadIdx.x < rg_multiples(Q)) {
+    uint32_t y[8] = {};
+    uint64_t carry = 0;
+#pragma unroll
+    for (int l = 0; l < L; ++l) {
+      carry += (uint64_t)threadIdx.x * T.P[l];
+      y[l] = (uint32_t)carry;
+      carry >>= 32;
+    }
+    uint4* const row = kP.v + threadIdx.x * (L == 4 ? 1 : 2);
+    row[0] = make_uint4(y[0], y[1], y[2], y[3]);
+    if (L == 5) row[1] = make_uint4(y[4], 0u, 0u, 0u);
   }
 }
 
@@ -600,7 +654,7 @@ template <int NT, int NP2, int NQ4, int QS = 256>
 __device__ __forceinline__ void rec4_groups(const OzTables& T, const uint4* kP, const uint32_t* wsm, int64_t i,
                                             int64_t j0, int64_t n, int32_t si, const int32_t* t,
                                             double* __restrict__ C, int64_t ldc) {
-  constexpr int Q = 3 * NT + 2 * NP2 + 4 * NQ4;
+  constexpr int Q = 3 * NT + 2 * NP2 + 4 * NQ4, L = rg_limbs(Q);
   int32_t tj[4];
   if (j0 + 4 <= n && (reinterpret_cast<uintptr_t>(t + j0) & 15) == 0) {
     const int4 v = ld_dep(reinterpret_cast<const int4*>(t + j0));
@@ -616,10 +670,10 @@ __device__ __forceinline__ void rec4_groups(const OzTables& T, const uint4* kP, 
   uint32_t slow = 0;
 #pragma unroll
   for (int e = 0; e < 4; ++e) {
-    uint32_t S[4];
+    uint32_t S[L];
     float f;
-    crt_groups<NT, NP2, NQ4>(T, w, e, S, f);
-    if (!round_groups_fast(kP, S, f, -(si + tj[e]), out[e])) slow |= 1u << e;
+    crt_groups<NT, NP2, NQ4, L>(T, w, e, S, f);
+    if (!round_groups_fast<L>(kP, rg_multiples(Q) - 1, S, f, -(si + tj[e]), out[e])) slow |= 1u << e;
   }
   if (slow) {                                              // rare: one branch for the four entries
 #pragma unroll
@@ -699,9 +753,9 @@ __global__ void __launch_bounds__(256, 2) reconstruct_groups_kernel(const __grid
                                                                     double* __restrict__ C, int64_t ldc,
                                                                     int64_t nch, int tpr_log2) {
   constexpr int Q = 3 * NT + 2 * NP2 + 4 * NQ4;
-  __shared__ uint4 kP[16];
+  __shared__ MultiplesOfP<Q> kPs;
   __shared__ uint32_t buf[2][Q * 256];
-  fill_kP(T, kP);
+  fill_kP<Q>(T, kPs);
   __syncthreads();
   pdl_wait();
   pdl_trigger();
@@ -724,7 +778,7 @@ __global__ void __launch_bounds__(256, 2) reconstruct_groups_kernel(const __grid
     cp_async_commit();
     cp_async_wait1();                       // this task's copies have landed
     const int64_t i = row_of(gi), j0 = col_of(c);
-    if (i < m && j0 < n) rec4_groups<NT, NP2, NQ4>(T, kP, mine + slot * Q * 256, i, j0, n, ld_dep(s + i), t, C, ldc);
+    if (i < m && j0 < n) rec4_groups<NT, NP2, NQ4>(T, kPs.v, mine + slot * Q * 256, i, j0, n, ld_dep(s + i), t, C, ldc);
     slot ^= 1;
     b = bn, gi = gn, c = cn;
   }
@@ -742,9 +796,9 @@ __global__ void __launch_bounds__(256, 2) reconstruct_groups8_kernel(const __gri
                                                                      double* __restrict__ C, int64_t ldc,
                                                                      int64_t nch, int tpr_log2) {
   constexpr int Q = 3 * NT + 2 * NP2 + 4 * NQ4;
-  __shared__ uint4 kP[16];
+  __shared__ MultiplesOfP<Q> kPs;
   extern __shared__ uint32_t dbuf[];
-  fill_kP(T, kP);
+  fill_kP<Q>(T, kPs);
   __syncthreads();
   pdl_wait();
   pdl_trigger();
@@ -771,8 +825,8 @@ __global__ void __launch_bounds__(256, 2) reconstruct_groups8_kernel(const __gri
     if (i < m && j0 < n) {
       const int32_t si = ld_dep(s + i);
       const uint32_t* w = mine + slot * Q * 512;
-      rec4_groups<NT, NP2, NQ4, 512>(T, kP, w, i, j0, n, si, t, C, ldc);
-      if (j0 + 4 < n) rec4_groups<NT, NP2, NQ4, 512>(T, kP, w + 1, i, j0 + 4, n, si, t, C, ldc);
+      rec4_groups<NT, NP2, NQ4, 512>(T, kPs.v, w, i, j0, n, si, t, C, ldc);
+      if (j0 + 4 < n) rec4_groups<NT, NP2, NQ4, 512>(T, kPs.v, w + 1, i, j0 + 4, n, si, t, C, ldc);
     }
     slot ^= 1;
     b = bn, gi = gn, c = cn;
@@ -790,24 +844,25 @@ __global__ void __launch_bounds__(256) reconstruct_groups_grouped_kernel(const _
                                                                          const OzGroupProblem* __restrict__ probs,
                                                                          const int32_t* __restrict__ map) {
   constexpr int Q = 3 * NT + 2 * NP2 + 4 * NQ4;
-  __shared__ uint4 kP[16];
+  __shared__ MultiplesOfP<Q> kPs;
   extern __shared__ uint32_t dbuf[];                   // [Q][256 threads][2 words]
-  fill_kP(T, kP);
-  __syncthreads();
   const int64_t b = blockIdx.x;
   const OzGroupProblem& P = probs[__ldg(map + b)];
   const int tpr = P.rec_tpr, rows = 256 / tpr;
   const int64_t l = b - P.rec_begin, nch = (P.n + 8 * tpr - 1) / (8 * tpr);
   const int64_t i = (l / nch) * rows + threadIdx.x / tpr;
   const int64_t j0 = ((l % nch) * tpr + threadIdx.x % tpr) * 8;
-  if (i >= P.m || j0 >= P.n) return;
+  const bool live = i < P.m && j0 < P.n;
   uint32_t* const mine = dbuf + 2 * threadIdx.x;
-  issue_digits8<Q>(P.Y, P.m * P.ldy, P.ldy, i, j0, P.n, mine);
+  if (live) issue_digits8<Q>(P.Y, P.m * P.ldy, P.ldy, i, j0, P.n, mine);
   cp_async_commit();
-  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  fill_kP<Q>(T, kPs);                                  // while the digits arrive
+  __syncthreads();
+  if (!live) return;
   const int32_t si = __ldg(P.s + i);
-  rec4_groups<NT, NP2, NQ4, 512>(T, kP, mine, i, j0, P.n, si, P.t, P.C, P.ldc);
-  if (j0 + 4 < P.n) rec4_groups<NT, NP2, NQ4, 512>(T, kP, mine + 1, i, j0 + 4, P.n, si, P.t, P.C, P.ldc);
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  rec4_groups<NT, NP2, NQ4, 512>(T, kPs.v, mine, i, j0, P.n, si, P.t, P.C, P.ldc);
+  if (j0 + 4 < P.n) rec4_groups<NT, NP2, NQ4, 512>(T, kPs.v, mine + 1, i, j0 + 4, P.n, si, P.t, P.C, P.ldc);
 }
 
 // Grouped: a block covers 256 / tpr rows of one column chunk of 4 tpr entries
@@ -901,11 +956,12 @@ cudaError_t launch_groups(const OzTables& T, int64_t m, int64_t n, const uint8_t
 }
 
 // The group shape of a plan (oz_plan.cpp, fill_group_tables), as a switch
-// over the shapes Q = 9 .. 16 give: -1 if the plan has none.
+// over the shapes Q = 9 .. 20 give: -1 if the plan has none.
 int group_shape(const OzTables& T) {
   const int key = T.rg_nt * 100 + T.rg_np2 * 10 + T.rg_nq4;
   switch (key) {
     case 300: case 220: case 310: case 400: case 301: case 320: case 410: case 500: case 401: case 420:
+    case 510: case 600: case 501: case 520: case 610:
       return key;
     default: return -1;
   }
@@ -924,6 +980,11 @@ cudaError_t with_shape(int key, F f) {
     case 500: return f(std::integral_constant<int, 5>(), std::integral_constant<int, 0>(), std::integral_constant<int, 0>());
     case 401: return f(std::integral_constant<int, 4>(), std::integral_constant<int, 0>(), std::integral_constant<int, 1>());
     case 420: return f(std::integral_constant<int, 4>(), std::integral_constant<int, 2>(), std::integral_constant<int, 0>());
+    case 510: return f(std::integral_constant<int, 5>(), std::integral_constant<int, 1>(), std::integral_constant<int, 0>());
+    case 600: return f(std::integral_constant<int, 6>(), std::integral_constant<int, 0>(), std::integral_constant<int, 0>());
+    case 501: return f(std::integral_constant<int, 5>(), std::integral_constant<int, 0>(), std::integral_constant<int, 1>());
+    case 520: return f(std::integral_constant<int, 5>(), std::integral_constant<int, 2>(), std::integral_constant<int, 0>());
+    case 610: return f(std::integral_constant<int, 6>(), std::integral_constant<int, 1>(), std::integral_constant<int, 0>());
     default: return cudaErrorInvalidValue;
   }
 }
