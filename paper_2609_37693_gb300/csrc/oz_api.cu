@@ -162,16 +162,16 @@ oz_status dgemm_run(oz_plan plan, int trans_a, int trans_b, int64_t m, int64_t n
     const oz::SplitOperand ob = {trans_b != 0, B, ldb, n, L.n_pad, t, V, colmax};
     e = oz::launch_split_both(T, oa, ob, k, L.k_pad, flag, st);
   } else {
-    e = trans_a ? oz::launch_split_cols(T, m, k, A, lda, L.m_pad, L.k_pad, s, U, bf16, flag, colmax, st)
-                : oz::launch_split_rows(T, m, k, A, lda, L.m_pad, L.k_pad, s, U, bf16, flag, st);
+    e = trans_a ? oz::launch_split_cols(T, m, k, A, lda, L.m_pad, L.k_pad, s, U, bf16, flag, colmax, st, false, !bf16)
+                : oz::launch_split_rows(T, m, k, A, lda, L.m_pad, L.k_pad, s, U, bf16, flag, st, false, !bf16);
     if (e == cudaSuccess && trans_b) {
-      e = oz::launch_split_rows(T, n, k, B, ldb, L.n_pad, L.k_pad, t, V, bf16, flag, st);
+      e = oz::launch_split_rows(T, n, k, B, ldb, L.n_pad, L.k_pad, t, V, bf16, flag, st, false, !bf16);
     } else if (e == cudaSuccess && bf16) {
-      e = oz::launch_split_cols(T, n, k, B, ldb, L.n_pad, L.k_pad, t, V, bf16, flag, colmax, st);
+      e = oz::launch_split_cols(T, n, k, B, ldb, L.n_pad, L.k_pad, t, V, bf16, flag, colmax, st, false, !bf16);
     } else if (e == cudaSuccess) {
       double* Bt = reinterpret_cast<double*>(ws + L.bt);
       e = oz::launch_transpose(k, n, B, ldb, Bt, st);
-      if (e == cudaSuccess) e = oz::launch_split_rows(T, n, k, Bt, k, L.n_pad, L.k_pad, t, V, bf16, flag, st);
+      if (e == cudaSuccess) e = oz::launch_split_rows(T, n, k, Bt, k, L.n_pad, L.k_pad, t, V, bf16, flag, st, false, !bf16);
     }
   }
   if (e != cudaSuccess) return OZ_ERR_CUDA;
@@ -280,11 +280,11 @@ extern "C" oz_status oz_dgemm_blocked(oz_plan plan, int trans_a, int trans_b, in
         e = oz::launch_gemm_fp(F, m, n, L.m_pad, L.n_pad, k_pad, U8, V8, reinterpret_cast<uint16_t*>(Y), L.ldy, mode,
                                flag, st);
     } else {
-      e = trans_a ? oz::launch_split_cols(T, m, len, As, lda, L.m_pad, k_pad, s, U, bf16, flag, colmax, st, true)
-                  : oz::launch_split_rows(T, m, len, As, lda, L.m_pad, k_pad, s, U, bf16, flag, st, true);
+      e = trans_a ? oz::launch_split_cols(T, m, len, As, lda, L.m_pad, k_pad, s, U, bf16, flag, colmax, st, true, !bf16)
+                  : oz::launch_split_rows(T, m, len, As, lda, L.m_pad, k_pad, s, U, bf16, flag, st, true, !bf16);
       if (e == cudaSuccess)
-        e = trans_b ? oz::launch_split_rows(T, n, len, Bs, ldb, L.n_pad, k_pad, t, V, bf16, flag, st, true)
-                    : oz::launch_split_cols(T, n, len, Bs, ldb, L.n_pad, k_pad, t, V, bf16, flag, colmax, st, true);
+        e = trans_b ? oz::launch_split_rows(T, n, len, Bs, ldb, L.n_pad, k_pad, t, V, bf16, flag, st, true, !bf16)
+                    : oz::launch_split_cols(T, n, len, Bs, ldb, L.n_pad, k_pad, t, V, bf16, flag, colmax, st, true, !bf16);
       if (e == cudaSuccess)
         e = plan->engine == OZ_ENGINE_TC1
                 ? oz::launch_gemm_tc_single(T, m, n, L.m_pad, L.n_pad, k_pad, U, V, Y, L.ldy, mode, flag, st)

@@ -64,9 +64,10 @@ constexpr int kSmemBytes = STAGES * STAGE_BYTES + kBarBytes + 1024;
 
 // Instruction descriptor of tcgen05.mma.kind::f16: D = F32 (bits 4-5 = 1),
 // A = B = BF16 (bits 7-9, 10-12 = 1), both K-major (bits 15, 16 = 0),
-// N >> 3 at bits 17-22, M >> 4 at bits 24-28.
-constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) |
-                            ((uint32_t)(BM >> 4) << 24);
+// N >> 3 at bits 17-22, M >> 4 at bits 24-28 (M = 256 across a pair).
+__host__ __device__ constexpr uint32_t idesc_bf16(int M, int N) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+}
 
 // ---- tcgen05 ----
 __device__ __forceinline__ void tmem_alloc(uint32_t dst_smem, uint32_t ncols) {
@@ -82,25 +83,24 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-__device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t accumulate) {
+__device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                          uint32_t accumulate) {
   asm volatile(
       "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
       " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
-      "l"(adesc), "l"(bdesc), "r"(kIdesc), "r"(accumulate)
+      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
 __device__ __forceinline__ void umma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
-// M = 256 across the pair (128 rows of A in each CTA), N = 256 (128 rows of B in each)
-constexpr uint32_t kIdescPair = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(256 >> 3) << 17) |
-                                ((uint32_t)(256 >> 4) << 24);
-__device__ __forceinline__ void umma_bf16_pair(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t accumulate) {
+__device__ __forceinline__ void umma_bf16_pair(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                               uint32_t accumulate) {
   asm volatile(
       "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
       " tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
-      "l"(adesc), "l"(bdesc), "r"(kIdescPair), "r"(accumulate)
+      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
 
@@ -135,6 +135,21 @@ __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.
 __device__ __forceinline__ uint64_t sdesc(uint32_t saddr) {
   return (uint64_t)((saddr >> 4) & 0x3FFFu) | ((uint64_t)1 << 16) | ((uint64_t)(1024 >> 4) << 32) |
          ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
+}
+
+// Columns of an output tile: the least multiple of 32 (a pair's N comes in
+// steps of 32) that covers n in ceil(n / 256) tiles, so that a ragged n does not
+// multiply, stage and drain up to 255 columns of padding (777 columns: four tiles
+// of 224 instead of 256).
+inline int tile_cols(int64_t n) {
+  const int64_t tiles = (n + BN - 1) / BN;
+  return (int)round_up((n + tiles - 1) / tiles, 32);
+}
+
+// Columns of a tile of bn that each of `groups` column groups of epilogue
+// warps takes: whole 32-column chunks, spread over the groups.
+__device__ __forceinline__ int cols_per_group(int bn, int groups) {
+  return ((bn + groups - 1) / groups + 31) & ~31;
 }
 
 struct Coord {
@@ -292,10 +307,11 @@ __device__ __forceinline__ void store_digits(uint8_t* dst, const uint32_t* w, in
 // the accumulator released at once (one arrival per warp), so that the
 // products of the unit after next start while this warp forms the digits
 // (W mod m reduced exactly, then the CRT digit, or W mod m when raw), one byte
-// per entry in acc8.
-template <int NCH, typename R>
-__device__ __forceinline__ void drain_one_slab(uint32_t taddr0, uint32_t (&acc8)[NCH * 8], const EpiConst& k,
-                                               R release) {
+// per entry in acc8. nch: this warp's 32-column chunks, at most two (a form each,
+// compiled apart: conditions on the chunks cost spills and 16 % at 65536 x 256 x
+// 256); without any, one is drained that is not stored.
+template <int NCH, int NW, typename R>
+__device__ __forceinline__ void drain_chunks(uint32_t taddr0, uint32_t (&acc8)[NW], const EpiConst& k, R release) {
   uint32_t v[NCH][32];
 #pragma unroll
   for (int ch = 0; ch < NCH; ++ch) tmem_ld32(taddr0 + ch * 32, v[ch]);
@@ -307,9 +323,18 @@ __device__ __forceinline__ void drain_one_slab(uint32_t taddr0, uint32_t (&acc8)
 #pragma unroll
     for (int w = 0; w < 8; ++w) acc8[ch * 8 + w] = bytes4(v[ch] + 4 * w, 0u, true, false, k);
 }
+template <typename R>
+__device__ __forceinline__ void drain_one_slab(uint32_t taddr0, int nch, uint32_t (&acc8)[16], const EpiConst& k,
+                                               R release) {
+  if (nch == 2)
+    drain_chunks<2>(taddr0, acc8, k, release);
+  else
+    drain_chunks<1>(taddr0, acc8, k, release);
+}
 
 struct Params {
   int m, n, tiles_m, tiles_n, num_tiles, kblocks, m_pad, n_pad, raw;
+  int bn;            // columns of a tile (tile_cols)
   uint8_t* Y;
   int64_t ldy;       // row pitch of Y
   int32_t* status;
@@ -404,12 +429,12 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       for (int t = blockIdx.x; t < num_units && ok; t += gridDim.x) {
         const Unit u = unit_of(p, t);
         const int ya = u.c.q * p.m_pad + u.c.tm * BM;
-        const int yb = u.c.q * p.n_pad + u.c.tn * BN;
+        const int yb = u.c.q * p.n_pad + u.c.tn * p.bn;
         for (int kb = u.kb0; kb < u.kb1; ++kb) {
           if (!mbar_wait(empty_bar(s), ph ^ 1u, abort_flag, p.status)) { ok = false; break; }
           outstanding[s] = false;
           const uint32_t sa = base + s * STAGE_BYTES;
-          mbar_expect_tx(full_bar(s), STAGE_BYTES);
+          mbar_expect_tx(full_bar(s), A_BYTES + p.bn * BK * 2);
           tma_load_2d(sa, &tmA, full_bar(s), kb * BK, ya);
           tma_load_2d(sa + A_BYTES, &tmB, full_bar(s), kb * BK, yb);
           outstanding[s] = true;
@@ -428,6 +453,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       int s = 0;
       uint32_t ph = 0;
       uint32_t g = 0;  // slab counter across tiles
+      const uint32_t idesc = idesc_bf16(BM, p.bn);
       bool ok = true;
       for (int t = blockIdx.x; t < num_units && ok; t += gridDim.x) {
         const Unit u = unit_of(p, t);
@@ -445,7 +471,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             const uint32_t sb = sa + A_BYTES;
 #pragma unroll
             for (int kk = 0; kk < BK / 16; ++kk)
-              umma_bf16(dtm, sdesc(sa + kk * 32), sdesc(sb + kk * 32), (sl >= 2 || kb > kb0 || kk > 0) ? 1u : 0u);
+              umma_bf16(dtm, sdesc(sa + kk * 32), sdesc(sb + kk * 32), idesc,
+                        (sl >= 2 || kb > kb0 || kk > 0) ? 1u : 0u);
             umma_commit(empty_bar(s));  // frees the stage once these products have read it
             if (++s == STAGES) { s = 0; ph ^= 1u; }
           }
@@ -466,7 +493,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     // and turns the last slab's sum into the digit in fp32.
     const int e = warp - 2;
     const int quarter = warp & 3;            // TMEM lanes 32*quarter .. +31
-    const int cbase = (e >> 2) * CPW1;       // columns cbase .. cbase + CPW1 - 1
+    const int cpw = cols_per_group(p.bn, kEpiWarps / 4);   // columns cbase .. cbase + cpw - 1, at most CPW1
+    const int cbase = (e >> 2) * cpw;
+    const int nch = cbase < p.bn ? min(cpw, p.bn - cbase) / 32 : 0;
     const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
     p.unmark(blockIdx.x * (kEpiWarps * 32) + threadIdx.x - 64, gridDim.x * (kEpiWarps * 32));
     uint32_t g = 0;
@@ -476,11 +505,15 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       const Coord c = u.c;
       const int nslabs = u.nslabs;
       const EpiConst k = epi_const((float)T.m[c.q], T.invm[c.q], p.raw ? 1.0f : (float)T.inv[c.q]);
-      const int row = c.tm * BM + quarter * 32 + lane;
-      const int col0 = c.tn * BN + cbase;
-      const bool in = row < p.m && col0 < p.n;
-      const bool runs = (p.ldy & 15) == 0 && (reinterpret_cast<uintptr_t>(p.Y) & 15) == 0;
-      uint8_t* const dst = p.Y + (size_t)u.ks * p.ysplit + (size_t)c.q * p.m * p.ldy + (size_t)row * p.ldy + col0;
+      // f(digits' place, how many of its columns are stored, whether in 16-byte runs) if this thread stores any
+      auto with_place = [&](auto f) {
+        const int row = c.tm * BM + quarter * 32 + lane;
+        const int col0 = c.tn * p.bn + cbase;
+        const int left = min(p.n - col0, nch * 32);
+        if (row < p.m && left > 0)
+          f(p.Y + (size_t)u.ks * p.ysplit + (size_t)c.q * p.m * p.ldy + (size_t)row * p.ldy + col0, left,
+            (p.ldy & 15) == 0 && (reinterpret_cast<uintptr_t>(p.Y) & 15) == 0);
+      };
       uint4 old[ACC ? CPW1 / 16 : 1];
       uint32_t acc8[CPW1 / 4];
 #pragma unroll
@@ -488,12 +521,13 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       for (int sl = 0; sl < nslabs; ++sl, ++g) {
         const uint32_t b = g & 1u, use = g >> 1;
         if constexpr (ACC)
-          if (sl + 1 == nslabs && in && runs) load_old_digits<CPW1 / 4>(old, dst, p.n - col0);
+          if (sl + 1 == nslabs)
+            with_place([&](uint8_t* dst, int left, bool runs) { if (runs) load_old_digits<CPW1 / 4>(old, dst, left); });
         if (!mbar_wait(tfull_bar(b), use & 1u, abort_flag, p.status)) { ok = false; break; }
         tc_fence_after();
         if constexpr (ONE) {
           const uint32_t tb = tempty_bar(b);
-          drain_one_slab<CPW1 / 32>(tmem_base + lane_addr + b * BN + cbase, acc8, k,
+          drain_one_slab(tmem_base + lane_addr + b * BN + cbase, nch, acc8, k,
                                     [&] {
                                       __syncwarp();
                                       if (lane == 0) mbar_arrive_relaxed(tb);
@@ -504,6 +538,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         const bool last = sl + 1 == nslabs;
 #pragma unroll
         for (int ch = 0; ch < CPW1 / 32; ++ch) {
+          if (ch >= nch) break;
           const uint32_t taddr = tmem_base + lane_addr + b * BN + cbase + ch * 32;
           uint32_t v[32];
           tmem_ld32(taddr, v);
@@ -523,7 +558,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       }
       if (!ok) break;
       // ---- tile done: acc8 holds the digits (or W mod m), one byte per entry ----
-      if (in) store_digits<CPW1 / 4>(dst, acc8, p.n - col0, runs, ACC, T.m[c.q], old);
+      with_place([&](uint8_t* dst, int left, bool runs) {
+        store_digits<CPW1 / 4>(dst, acc8, left, runs, ACC, T.m[c.q], old);
+      });
     }
   }
 
@@ -575,6 +612,7 @@ struct PairUnit {
   uint8_t* Y;               // digit plane of this unit (row pitch ldy, m rows, n columns)
   int64_t ldy;
   int m, n, row0, col0;     // the output's size and the tile's first row and column
+  int bn;                   // the tile's columns
   int raw;
 };
 
@@ -596,7 +634,7 @@ struct PairSingle {
     w.mA = &mapA;
     w.mB = &mapB;
     w.ya = u.c.q * p.m_pad + u.c.tm * 2 * P_BM;
-    w.yb = u.c.q * p.n_pad + u.c.tn * 2 * P_BN;
+    w.yb = u.c.q * p.n_pad + u.c.tn * p.bn;
     w.kb0 = u.kb0;
     w.kb1 = u.kb1;
     w.nslabs = u.nslabs;
@@ -606,7 +644,8 @@ struct PairSingle {
     w.m = p.m;
     w.n = p.n;
     w.row0 = u.c.tm * 2 * P_BM;
-    w.col0 = u.c.tn * 2 * P_BN;
+    w.col0 = u.c.tn * p.bn;
+    w.bn = p.bn;
     w.raw = p.raw;
     return w;
   }
@@ -637,7 +676,7 @@ struct PairGrouped {
     w.mA = &P.mapA;
     w.mB = &P.mapB;
     w.ya = c.q * (int)P.m_pad + c.tm * 2 * P_BM;
-    w.yb = c.q * (int)P.n_pad + c.tn * 2 * P_BN;
+    w.yb = c.q * (int)P.n_pad + c.tn * P.bn;
     w.kb0 = 0;
     w.kb1 = P.kblocks;
     w.nslabs = (P.kblocks + kSlabBlocks - 1) / kSlabBlocks;
@@ -647,14 +686,15 @@ struct PairGrouped {
     w.m = (int)P.m;
     w.n = (int)P.n;
     w.row0 = c.tm * 2 * P_BM;
-    w.col0 = c.tn * 2 * P_BN;
+    w.col0 = c.tn * P.bn;
+    w.bn = P.bn;
     w.raw = 0;
     return w;
   }
 };
 
 // EW epilogue warps: every warp drains the 32 TMEM lanes of its quarter (warp
-// index mod 4), over CPW = 256 / (EW / 4) columns.
+// index mod 4), over at most CPW = 256 / (EW / 4) columns.
 // S: the unit scheduler (PairSingle or PairGrouped).
 template <int EW, typename S, bool ONE, bool ACC>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__((2 + EW) * 32, 1)
@@ -721,12 +761,13 @@ gemm_tc_pair_kernel(const __grid_constant__ S sched, const __grid_constant__ OzT
       for (int t = pair; t < num_units && ok; t += npairs) {
         const PairUnit u = sched.unit(t, pi);
         const int ya = u.ya + (int)rank * P_BM;
-        const int yb = u.yb + (int)rank * P_BN;
+        const int yb = u.yb + (int)rank * (u.bn / 2);
+        const uint32_t bytes = 2u * (P_A_BYTES + (uint32_t)u.bn * BK);   // both CTAs' A, half of B's rows each
         for (int kb = u.kb0; kb < u.kb1; ++kb) {
           if (!mbar_wait(empty_bar(s), ph ^ 1u, abort_flag, status)) { ok = false; break; }
           outstanding[s] = false;
           const uint32_t sa = base + s * P_STAGE_BYTES;
-          if (leader) mbar_expect_tx(full_bar(s), 2 * P_STAGE_BYTES);
+          if (leader) mbar_expect_tx(full_bar(s), bytes);
           const uint32_t fb = mapa(full_bar(s), 0);
           tma_load_2d_pair(sa, u.mA, fb, kb * BK, ya);
           tma_load_2d_pair(sa + P_A_BYTES, u.mB, fb, kb * BK, yb);
@@ -752,6 +793,7 @@ gemm_tc_pair_kernel(const __grid_constant__ S sched, const __grid_constant__ OzT
       int pi = sched.first(pair);
       for (int t = pair; t < num_units && ok; t += npairs) {
         const PairUnit u = sched.unit(t, pi);
+        const uint32_t idesc = idesc_bf16(2 * P_BM, u.bn);
         for (int sl = 0; sl < u.nslabs && ok; ++sl, ++g) {
           const uint32_t b = g & 1u, use = g >> 1;
           if (!mbar_wait(tempty_bar(b), (use & 1u) ^ 1u, abort_flag, status)) { ok = false; break; }
@@ -766,7 +808,8 @@ gemm_tc_pair_kernel(const __grid_constant__ S sched, const __grid_constant__ OzT
             const uint32_t sb = sa + P_A_BYTES;
 #pragma unroll
             for (int kk = 0; kk < BK / 16; ++kk)
-              umma_bf16_pair(dtm, sdesc(sa + kk * 32), sdesc(sb + kk * 32), (sl >= 2 || kb > kb0 || kk > 0) ? 1u : 0u);
+              umma_bf16_pair(dtm, sdesc(sa + kk * 32), sdesc(sb + kk * 32), idesc,
+                             (sl >= 2 || kb > kb0 || kk > 0) ? 1u : 0u);
             umma_commit_pair_both(empty_bar(s));
             if (++s == P_STAGES) { s = 0; ph ^= 1u; }
           }
@@ -790,7 +833,6 @@ gemm_tc_pair_kernel(const __grid_constant__ S sched, const __grid_constant__ OzT
     // the 32 TMEM lanes of its quarter (warp index mod 4) over CPW columns.
     const int e = warp - 2;
     const int quarter = warp & 3;
-    const int cbase = (e >> 2) * CPW;          // first column this warp drains
     const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
     sched.unmark((int)blockIdx.x * (EW * 32) + (int)threadIdx.x - 64, (int)gridDim.x * (EW * 32));
     uint32_t g = 0;
@@ -800,11 +842,18 @@ gemm_tc_pair_kernel(const __grid_constant__ S sched, const __grid_constant__ OzT
       const PairUnit u = sched.unit(t, pi);
       const int nslabs = u.nslabs;
       const EpiConst k = epi_const((float)T.m[u.q], T.invm[u.q], u.raw ? 1.0f : (float)T.inv[u.q]);
-      const int row = u.row0 + (int)rank * P_BM + quarter * 32 + lane;
-      const int col0 = u.col0 + cbase;
-      const bool in = row < u.m && col0 < u.n;
-      const bool runs = (u.ldy & 15) == 0 && (reinterpret_cast<uintptr_t>(u.Y) & 15) == 0;
-      uint8_t* const dst = u.Y + (size_t)row * u.ldy + col0;
+      const int cpw = cols_per_group(u.bn, EW / 4);   // this warp's columns: cbase .. cbase + cpw - 1, at most CPW
+      const int cbase = (e >> 2) * cpw;
+      const int nch = cbase < u.bn ? min(cpw, u.bn - cbase) / 32 : 0;
+      // as in gemm_tc_kernel
+      auto with_place = [&](auto f) {
+        const int row = u.row0 + (int)rank * P_BM + quarter * 32 + lane;
+        const int col0 = u.col0 + cbase;
+        const int left = min(u.n - col0, nch * 32);
+        if (row < u.m && left > 0)
+          f(u.Y + (size_t)row * u.ldy + col0, left,
+            (u.ldy & 15) == 0 && (reinterpret_cast<uintptr_t>(u.Y) & 15) == 0);
+      };
       uint4 old[ACC ? CPW / 16 : 1];
       uint32_t acc8[CPW / 4];                // residue + 128 of the chain of slab nsl - 2, one byte per column
 #pragma unroll
@@ -812,12 +861,13 @@ gemm_tc_pair_kernel(const __grid_constant__ S sched, const __grid_constant__ OzT
       for (int sl = 0; sl < nslabs; ++sl, ++g) {
         const uint32_t b = g & 1u, use = g >> 1;
         if constexpr (ACC)
-          if (sl + 1 == nslabs && in && runs) load_old_digits<CPW / 4>(old, dst, u.n - col0);
+          if (sl + 1 == nslabs)
+            with_place([&](uint8_t* dst, int left, bool runs) { if (runs) load_old_digits<CPW / 4>(old, dst, left); });
         if (!mbar_wait(tfull_bar(b), use & 1u, abort_flag, status)) { ok = false; break; }
         tc_fence_after();
         if constexpr (ONE) {
           const uint32_t tb = mapa(tempty_bar(b), 0);
-          drain_one_slab<CPW / 32>(tmem_base + lane_addr + b * 256 + cbase, acc8, k,
+          drain_one_slab(tmem_base + lane_addr + b * 256 + cbase, nch, acc8, k,
                                    [&] {
                                      __syncwarp();
                                      if (lane == 0) mbar_arrive_cluster(tb);
@@ -828,6 +878,7 @@ gemm_tc_pair_kernel(const __grid_constant__ S sched, const __grid_constant__ OzT
         const bool last = sl + 1 == nslabs;
 #pragma unroll
         for (int ch = 0; ch < CPW / 32; ++ch) {
+          if (ch >= nch) break;
           const uint32_t taddr = tmem_base + lane_addr + b * 256 + cbase + ch * 32;
           uint32_t v[32];
           tmem_ld32(taddr, v);
@@ -847,7 +898,9 @@ gemm_tc_pair_kernel(const __grid_constant__ S sched, const __grid_constant__ OzT
       }
       if (!ok) break;
       // ---- tile done: acc8 holds the digits (or W mod m), one byte per entry ----
-      if (in) store_digits<CPW / 4>(dst, acc8, u.n - col0, runs, ACC, T.m[u.q], old);
+      with_place([&](uint8_t* dst, int left, bool runs) {
+        store_digits<CPW / 4>(dst, acc8, left, runs, ACC, T.m[u.q], old);
+      });
     }
   }
 
@@ -931,12 +984,12 @@ gemm_tc_grouped_kernel(const __grid_constant__ OzTables T, const OzGroupProblem*
         const OzGroupProblem& P = probs[pi];
         const Coord c = tile_coord((int)(t - P.unit_begin), P.tiles_m, P.tiles_n);
         const int ya = c.q * (int)P.m_pad + c.tm * BM;
-        const int yb = c.q * (int)P.n_pad + c.tn * BN;
+        const int yb = c.q * (int)P.n_pad + c.tn * P.bn;
         for (int kb = 0; kb < P.kblocks; ++kb) {
           if (!mbar_wait(empty_bar(s), ph ^ 1u, abort_flag, status)) { ok = false; break; }
           outstanding[s] = false;
           const uint32_t sa = base + s * STAGE_BYTES;
-          mbar_expect_tx(full_bar(s), STAGE_BYTES);
+          mbar_expect_tx(full_bar(s), A_BYTES + P.bn * BK * 2);
           tma_load_2d(sa, &P.mapA, full_bar(s), kb * BK, ya);
           tma_load_2d(sa + A_BYTES, &P.mapB, full_bar(s), kb * BK, yb);
           outstanding[s] = true;
@@ -962,6 +1015,7 @@ gemm_tc_grouped_kernel(const __grid_constant__ OzTables T, const OzGroupProblem*
         const OzGroupProblem& P = probs[pi];
         const int kblocks = P.kblocks;
         const int nslabs = (kblocks + kSlabBlocks - 1) / kSlabBlocks;
+        const uint32_t idesc = idesc_bf16(BM, P.bn);
         for (int sl = 0; sl < nslabs && ok; ++sl, ++g) {
           const uint32_t b = g & 1u, use = g >> 1;
           if (!mbar_wait(tempty_bar(b), (use & 1u) ^ 1u, abort_flag, status)) { ok = false; break; }
@@ -976,7 +1030,8 @@ gemm_tc_grouped_kernel(const __grid_constant__ OzTables T, const OzGroupProblem*
             const uint32_t sb = sa + A_BYTES;
 #pragma unroll
             for (int kk = 0; kk < BK / 16; ++kk)
-              umma_bf16(dtm, sdesc(sa + kk * 32), sdesc(sb + kk * 32), (sl >= 2 || kb > kb0 || kk > 0) ? 1u : 0u);
+              umma_bf16(dtm, sdesc(sa + kk * 32), sdesc(sb + kk * 32), idesc,
+                        (sl >= 2 || kb > kb0 || kk > 0) ? 1u : 0u);
             umma_commit(empty_bar(s));
             if (++s == STAGES) { s = 0; ph ^= 1u; }
           }
@@ -993,7 +1048,6 @@ gemm_tc_grouped_kernel(const __grid_constant__ OzTables T, const OzGroupProblem*
     // ------------------------------ epilogue ------------------------------
     const int e = warp - 2;
     const int quarter = warp & 3;
-    const int cbase = (e >> 2) * CPW1;
     const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
     uint32_t g = 0;
     bool ok = true;
@@ -1004,6 +1058,8 @@ gemm_tc_grouped_kernel(const __grid_constant__ OzTables T, const OzGroupProblem*
       const Coord c = tile_coord((int)(t - P.unit_begin), P.tiles_m, P.tiles_n);
       const int nslabs = (P.kblocks + kSlabBlocks - 1) / kSlabBlocks;
       const EpiConst k = epi_const((float)T.m[c.q], T.invm[c.q], (float)T.inv[c.q]);
+      const int cpw = cols_per_group(P.bn, kEpiWarps / 4), cbase = (e >> 2) * cpw;
+      const int nch = cbase < P.bn ? min(cpw, P.bn - cbase) / 32 : 0;
       uint32_t acc8[CPW1 / 4];
 #pragma unroll
       for (int i = 0; i < CPW1 / 4; ++i) acc8[i] = 0x80808080u;
@@ -1013,7 +1069,7 @@ gemm_tc_grouped_kernel(const __grid_constant__ OzTables T, const OzGroupProblem*
         tc_fence_after();
         if constexpr (ONE) {
           const uint32_t tb = tempty_bar(b);
-          drain_one_slab<CPW1 / 32>(tmem_base + lane_addr + b * BN + cbase, acc8, k,
+          drain_one_slab(tmem_base + lane_addr + b * BN + cbase, nch, acc8, k,
                                     [&] {
                                       __syncwarp();
                                       if (lane == 0) mbar_arrive_relaxed(tb);
@@ -1024,6 +1080,7 @@ gemm_tc_grouped_kernel(const __grid_constant__ OzTables T, const OzGroupProblem*
         const bool last = sl + 1 == nslabs;
 #pragma unroll
         for (int ch = 0; ch < CPW1 / 32; ++ch) {
+          if (ch >= nch) break;
           const uint32_t taddr = tmem_base + lane_addr + b * BN + cbase + ch * 32;
           uint32_t v[32];
           tmem_ld32(taddr, v);
@@ -1043,11 +1100,12 @@ gemm_tc_grouped_kernel(const __grid_constant__ OzTables T, const OzGroupProblem*
       }
       if (!ok) break;
       const int row = c.tm * BM + quarter * 32 + lane;
-      const int col0 = c.tn * BN + cbase;
-      if (row < P.m && col0 < P.n) {
+      const int col0 = c.tn * P.bn + cbase;
+      const int left = (int)min(P.n - col0, (int64_t)(nch * 32));
+      if (row < P.m && left > 0) {
         uint8_t* dst = P.Y + (size_t)c.q * P.m * P.ldy + (size_t)row * P.ldy + col0;
-        store_digits<CPW1 / 4>(dst, acc8, P.n - col0, (P.ldy & 15) == 0 && (reinterpret_cast<uintptr_t>(P.Y) & 15) == 0,
-                               0, T.m[c.q], nullptr);
+        store_digits<CPW1 / 4>(dst, acc8, left, (P.ldy & 15) == 0 && (reinterpret_cast<uintptr_t>(P.Y) & 15) == 0, 0,
+                               T.m[c.q], nullptr);
       }
     }
   }
@@ -1126,7 +1184,7 @@ cudaError_t launch_gemm_tc(const OzTables& t, int64_t m, int64_t n, int64_t m_pa
     return cudaErrorInvalidValue;
   CUtensorMap mapA, mapB;
   if (!make_map(&mapA, U, (int64_t)t.Q * m_pad, k_pad, P_BM)) return cudaErrorInvalidValue;
-  if (!make_map(&mapB, V, (int64_t)t.Q * n_pad, k_pad, P_BN)) return cudaErrorInvalidValue;
+  if (!make_map(&mapB, V, (int64_t)t.Q * n_pad, k_pad, tile_cols(n) / 2)) return cudaErrorInvalidValue;
   int dev = 0, sms = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
@@ -1158,6 +1216,7 @@ cudaError_t launch_gemm_tc(const OzTables& t, int64_t m, int64_t n, int64_t m_pa
   p.n = (int)n;
   p.tiles_m = (int)tiles_m;
   p.tiles_n = (int)tiles_n;
+  p.bn = tile_cols(n);
   p.num_tiles = (int)num_tiles;
   p.kblocks = (int)(k_pad / BK);
   p.m_pad = (int)m_pad;
@@ -1173,12 +1232,14 @@ cudaError_t launch_gemm_tc(const OzTables& t, int64_t m, int64_t n, int64_t m_pa
   return launch_pdl(kernel, dim3((unsigned)(2 * pairs)), dim3((2 + epi_warps) * 32), (size_t)smem_bytes, st, 1, sched, t);
 }
 
-// Tensor maps of one grouped problem's planes (rows of Q planes): 128-row
-// boxes for A; for B 128-row boxes (CTA pairs) or 256-row boxes (the one-CTA
-// kernel).
+// Tensor maps of one grouped problem's planes (rows of Q planes) and its
+// tiles' columns: 128-row boxes for A; for B boxes of half a tile's columns (CTA
+// pairs) or of all (the one-CTA kernel).
 bool group_maps_tc(OzGroupProblem* pr, int Q, bool pairs) {
+  pr->bn = tile_cols(pr->n);
   return make_map(&pr->mapA, pr->U, (int64_t)Q * pr->m_pad, pr->k_pad, BM) &&
-         make_map(&pr->mapB, pr->V, (int64_t)Q * pr->n_pad, pr->k_pad, pairs ? P_BN : BN);
+         make_map(&pr->mapB, pr->V, (int64_t)Q * pr->n_pad, pr->k_pad,
+                  pairs ? pr->bn / 2 : pr->bn);
 }
 
 cudaError_t launch_gemm_tc_grouped(const OzTables& t, const OzGroupProblem* probs, int count, int64_t total_units,
@@ -1233,7 +1294,7 @@ cudaError_t launch_gemm_tc_single(const OzTables& t, int64_t m, int64_t n, int64
     return cudaErrorInvalidValue;
   CUtensorMap mapA, mapB;
   if (!make_map(&mapA, U, (int64_t)t.Q * m_pad, k_pad, BM)) return cudaErrorInvalidValue;
-  if (!make_map(&mapB, V, (int64_t)t.Q * n_pad, k_pad, BN)) return cudaErrorInvalidValue;
+  if (!make_map(&mapB, V, (int64_t)t.Q * n_pad, k_pad, tile_cols(n))) return cudaErrorInvalidValue;
   int dev = 0, sms = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
@@ -1249,6 +1310,7 @@ cudaError_t launch_gemm_tc_single(const OzTables& t, int64_t m, int64_t n, int64
   p.n = (int)n;
   p.tiles_m = (int)tiles_m;
   p.tiles_n = (int)tiles_n;
+  p.bn = tile_cols(n);
   p.num_tiles = (int)num_tiles;
   p.kblocks = (int)(k_pad / BK);
   p.m_pad = (int)m_pad;

@@ -102,11 +102,11 @@ Blocks blocks_of(const Part& P, int64_t m, int64_t n, int64_t k, int ept) {
   // one block per row, else one warp per row (eight rows per block: fewer,
   // fuller blocks on the short and middling rows of a batch)
   const bool long_rows = P.k_pad > 4096;
-  b.rows = long_rows ? P.m_pad : 0;
-  b.wrows = long_rows ? 0 : P.m_pad / 8;
+  b.rows = long_rows ? m : 0;                // plane rows past m or n are not written
+  b.wrows = long_rows ? 0 : (m + 7) / 8;
   b.cm = ((n + 31) / 32) * ((k + 255) / 256);
   b.sh = (n + 255) / 256;
-  b.sc = (P.n_pad / 32) * (P.k_pad / 64);
+  b.sc = ((n + 31) / 32) * (P.k_pad / 64);
   const int tpr = rec_tpr(n, ept);
   b.rec = ((m + 256 / tpr - 1) / (256 / tpr)) * ((n + ept * (int64_t)tpr - 1) / (ept * (int64_t)tpr));
   return b;

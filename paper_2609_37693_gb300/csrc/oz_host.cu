@@ -200,7 +200,7 @@ extern "C" oz_status oz_dgemm_host(oz_plan plan, int64_t m, int64_t n, int64_t k
   double* Bt = reinterpret_cast<double*>(ws + L.bt);
   auto launch_split_b_chunk = [&](int64_t nc, int64_t c0, void* planes) {
     if (bf16) return oz::launch_split_cols(T, nc, k, Bd + c0, n, L.w_pad, L.k_pad, t + c0, planes, bf16, flag,
-                                           colmax + c0, sc);
+                                           colmax + c0, sc, false, false);
     cudaError_t r = oz::launch_transpose(k, nc, Bd + c0, n, Bt, sc);
     if (r != cudaSuccess) return r;
     return oz::launch_split_rows(T, nc, k, Bt, k, L.w_pad, L.k_pad, t + c0, planes, bf16, flag, sc);
@@ -214,7 +214,7 @@ extern "C" oz_status oz_dgemm_host(oz_plan plan, int64_t m, int64_t n, int64_t k
     if (k > 0)
       chk(fp ? oz::launch_split_fp(T, F, 1, nr, k, Ad[slot], k, L.chunk_pad, L.k_pad, s + r0,
                                    static_cast<uint8_t*>(U), flag, nullptr, sc)
-             : oz::launch_split_rows(T, nr, k, Ad[slot], k, L.chunk_pad, L.k_pad, s + r0, U, bf16, flag, sc));
+             : oz::launch_split_rows(T, nr, k, Ad[slot], k, L.chunk_pad, L.k_pad, s + r0, U, bf16, flag, sc, false, !bf16));
     chk(cudaEventRecord(ev_a_free[slot], sc));
     if (i + 2 < nbi) copy_a(i + 2);
     for (int64_t j = 0; j < nbj && e == cudaSuccess; ++j, ++blk) {

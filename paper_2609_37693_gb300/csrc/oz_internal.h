@@ -121,13 +121,14 @@ struct OzGroupProblem {
   int32_t* t;
   uint64_t* colmax;
   int32_t* flag;
-  int64_t rows_begin;   // split of A: one block per row of m_pad
+  int64_t rows_begin;   // split of A: one block per row of m (or per eight)
   int64_t cm_begin;     // column maxima of B: ceil(n/32) * ceil(k/256) blocks
   int64_t sh_begin;     // shifts of B: ceil(n/256) blocks
-  int64_t sc_begin;     // split of B: (n_pad/32) * (k_pad/64) blocks
+  int64_t sc_begin;     // split of B: ceil(n/32) * (k_pad/64) blocks
   int64_t unit_begin;   // GEMMs: Q * tiles_m * tiles_n units
   int64_t rec_begin;    // reconstruct: m * ceil(n/1024) blocks
   int tiles_m, tiles_n, kblocks;
+  int bn;               // columns of an output tile (at most 256)
   int rec_tpr;          // reconstruct: threads per row chunk (8..32), 256 / rec_tpr rows per block, each
                         // thread 8 entries (the groups' kernel) or 4 (the pairs')
 };
@@ -208,12 +209,15 @@ inline int64_t round_up(int64_t x, int64_t r) { return (x + r - 1) / r * r; }
 // Launchers (defined in the .cu files). Each returns cudaGetLastError().
 // given: the shifts are already in `shifts` (taken over a longer vector, as
 // in a blocked call); the split then neither scans for the maximum nor flags.
+// pad: write zeros to the bf16 plane rows past nvec (oz_split states them). The
+// products leave them as they are: such a row only reaches outputs past m or n,
+// which are not stored.
 cudaError_t launch_split_rows(const OzTables& t, int64_t nvec, int64_t len, const double* X, int64_t ld,
                               int64_t nvec_pad, int64_t k_pad, int32_t* shifts, void* planes, int bf16,
-                              int32_t* flag, cudaStream_t st, bool given = false);
+                              int32_t* flag, cudaStream_t st, bool given = false, bool pad = true);
 cudaError_t launch_split_cols(const OzTables& t, int64_t nvec, int64_t len, const double* X, int64_t ld,
                               int64_t nvec_pad, int64_t k_pad, int32_t* shifts, void* planes, int bf16,
-                              int32_t* flag, uint64_t* colmax, cudaStream_t st, bool given = false);
+                              int32_t* flag, uint64_t* colmax, cudaStream_t st, bool given = false, bool pad = true);
 // Both operands' shifts and bf16 planes in one or two launches, which also
 // clear the status word; vectors with a non-finite entry get a marked shift (kBadMark)
 // that the TC GEMM kernels unmark and report (their shifts argument).

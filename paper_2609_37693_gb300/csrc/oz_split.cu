@@ -307,9 +307,10 @@ __device__ __forceinline__ void split_row_warp(const OzTables& T, int64_t v, int
                                                const double* __restrict__ X, int64_t ld, int64_t nvec_pad,
                                                int64_t k_pad, int32_t* __restrict__ shifts,
                                                void* __restrict__ planes, int32_t* __restrict__ flag, bool given,
-                                               bool mark = false) {
+                                               bool pad, bool mark = false) {
   const int lane = threadIdx.x & 31;
   const bool live = v < nvec;
+  if (!live && !pad) return;          // the whole warp shares v
   const uint64_t* row = reinterpret_cast<const uint64_t*>(X) + (live ? v * ld : 0);
   int32_t s;
   if (given) {
@@ -358,9 +359,9 @@ __global__ void __launch_bounds__(256, NP > 5 ? 2 : 3) split_rows_warp_kernel(co
                                                               int64_t nvec_pad, int64_t k_pad,
                                                               int32_t* __restrict__ shifts,
                                                               void* __restrict__ planes, int32_t* __restrict__ flag,
-                                                              bool given) {
+                                                              bool given, bool pad) {
   const int64_t v = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
-  split_row_warp<kBF16, NP, QT>(T, v, nvec, len, X, ld, nvec_pad, k_pad, shifts, planes, flag, given);
+  split_row_warp<kBF16, NP, QT>(T, v, nvec, len, X, ld, nvec_pad, k_pad, shifts, planes, flag, given, pad);
 }
 
 // Grouped, short rows: block b holds rows 8 (b - rows_begin) .. + 7 of its
@@ -373,7 +374,7 @@ __global__ void __launch_bounds__(256, (QT > 0 && NP == 4) ? 3 : 2) split_rows_w
   const int64_t b = blockIdx.x;
   const OzGroupProblem& P = probs[__ldg(map + b)];
   const int64_t v = (b - P.rows_begin) * 8 + (threadIdx.x >> 5);
-  split_row_warp<true, NP, QT>(T, v, P.m, P.k, P.A, P.lda, P.m_pad, P.k_pad, P.s, P.U, P.flag, false);
+  split_row_warp<true, NP, QT>(T, v, P.m, P.k, P.A, P.lda, P.m_pad, P.k_pad, P.s, P.U, P.flag, false, false);
 }
 
 template <bool kBF16, int NP, int QT>
@@ -576,10 +577,11 @@ __device__ __forceinline__ void load_col8(const uint64_t* Xb, int64_t ld, bool l
   for (int e = 0; e < 8; ++e) b[e] = (live && h0 + e < len) ? ld_dep(Xb + (h0 + e) * ld + j) : 0ull;
 }
 
-// One tile from the entries b of this thread (lane's vector, shift s).
+// One tile from the entries b of this thread (lane's vector, shift s), vectors
+// below nstore.
 template <int NP, int QT>
 __device__ __forceinline__ void split_cols_entries(const OzTables& T, uint64_t (&b)[8], int32_t s, int64_t j0,
-                                                   int64_t hbase, int64_t nvec_pad, int64_t k_pad,
+                                                   int64_t hbase, int64_t nstore, int64_t nvec_pad, int64_t k_pad,
                                                    uint16_t* __restrict__ planes, uint32_t* tile) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   Pieces<NP> P[8];
@@ -603,7 +605,7 @@ __device__ __forceinline__ void split_cols_entries(const OzTables& T, uint64_t (
   __syncthreads();
   // thread t: vector row t / 8 of the tile, 16-byte chunk t % 8 of its 64 h
   const int row = threadIdx.x >> 3, ch = threadIdx.x & 7;
-  if (j0 + row < nvec_pad) {
+  if (j0 + row < nstore) {
     const int64_t plane = nvec_pad * k_pad;
     uint16_t* dst = planes + (j0 + row) * k_pad + hbase + 8 * ch;
     const uint4* src = reinterpret_cast<const uint4*>(tile + row * kColPitchWords + 4 * ch);
@@ -616,29 +618,30 @@ __device__ __forceinline__ void split_cols_entries(const OzTables& T, uint64_t (
 template <int NP, int QT>
 __device__ __forceinline__ void split_cols_tile(const OzTables& T, int64_t j0, int64_t hbase, int64_t nvec,
                                                 int64_t len, const double* __restrict__ X, int64_t ld,
-                                                int64_t nvec_pad, int64_t k_pad, const int32_t* __restrict__ shifts,
-                                                uint16_t* __restrict__ planes, uint32_t* tile) {
+                                                int64_t nstore, int64_t nvec_pad, int64_t k_pad,
+                                                const int32_t* __restrict__ shifts, uint16_t* __restrict__ planes,
+                                                uint32_t* tile) {
   const int64_t j = j0 + (threadIdx.x & 31);
   const bool live = j < nvec;
   const int32_t s = live ? __ldg(shifts + j) : 0;
   uint64_t b[8];
   load_col8(reinterpret_cast<const uint64_t*>(X), ld, live, j, hbase + 8 * (threadIdx.x >> 5), len, b);
-  split_cols_entries<NP, QT>(T, b, s, j0, hbase, nvec_pad, k_pad, planes, tile);
+  split_cols_entries<NP, QT>(T, b, s, j0, hbase, nstore, nvec_pad, k_pad, planes, tile);
 }
 
 template <int NP, int QT>
 __global__ void __launch_bounds__(256, NP > 5 ? 2 : 3) split_cols_bf16_kernel(const __grid_constant__ OzTables T, int64_t nvec,
                                                                 int64_t len, const double* __restrict__ X, int64_t ld,
-                                                                int64_t nvec_pad, int64_t k_pad,
+                                                                int64_t nstore, int64_t nvec_pad, int64_t k_pad,
                                                                 const int32_t* __restrict__ shifts,
                                                                 uint16_t* __restrict__ planes) {
   extern __shared__ uint4 col_tile[];
   split_cols_tile<NP, QT>(T, (int64_t)blockIdx.x * kColTileJ, (int64_t)blockIdx.y * kColTileH, nvec, len, X, ld,
-                          nvec_pad, k_pad, shifts, planes, reinterpret_cast<uint32_t*>(col_tile));
+                          nstore, nvec_pad, k_pad, shifts, planes, reinterpret_cast<uint32_t*>(col_tile));
 }
 
 // Grouped: block b is tile l = b - sc_begin of its problem's
-// (n_pad / 32) x (k_pad / 64) grid, vectors fastest; map[b] is its problem.
+// ceil(n / 32) x (k_pad / 64) grid, vectors fastest; map[b] is its problem.
 template <int NP, int QT>
 __global__ void __launch_bounds__(256, 3) split_cols_grouped_kernel(const __grid_constant__ OzTables T,
                                                                    const OzGroupProblem* __restrict__ probs,
@@ -646,8 +649,8 @@ __global__ void __launch_bounds__(256, 3) split_cols_grouped_kernel(const __grid
   extern __shared__ uint4 col_tile[];
   const int64_t b = blockIdx.x;
   const OzGroupProblem& P = probs[__ldg(map + b)];
-  const int64_t l = b - P.sc_begin, nbx = P.n_pad / kColTileJ;
-  split_cols_tile<NP, QT>(T, (l % nbx) * kColTileJ, (l / nbx) * kColTileH, P.n, P.k, P.B, P.ldb, P.n_pad, P.k_pad,
+  const int64_t l = b - P.sc_begin, nbx = (P.n + kColTileJ - 1) / kColTileJ;
+  split_cols_tile<NP, QT>(T, (l % nbx) * kColTileJ, (l / nbx) * kColTileH, P.n, P.k, P.B, P.ldb, P.n, P.n_pad, P.k_pad,
                           P.t, static_cast<uint16_t*>(P.V), reinterpret_cast<uint32_t*>(col_tile));
 }
 
@@ -678,7 +681,7 @@ struct SplitSide {
   uint16_t* planes;
   uint64_t* colmax;      // kSideTile: zeroed before the first launch
   int kind;              // kSideRow, kSideWarp, kSideStrip or kSideTile
-  int blocks1, blocks2;  // rows, strips (a multiple of kStripCtas) or maxima; tiles
+  int blocks1, blocks2;  // rows and strips (a multiple of kStripCtas) or maxima; tiles
 };
 constexpr int kSideRow = 0, kSideWarp = 1, kSideStrip = 2, kSideTile = 3, kSideAny = -1;
 constexpr int kStripCtas = 8;
@@ -740,7 +743,7 @@ __device__ __forceinline__ void split_strip(const OzTables& T, const SplitSide& 
   const int32_t s = sh[lane];
   for (int i = last; i >= 0; i -= kStripCtas) {
     if (i != last) load_col8(Xb, S.ld, live, j, (int64_t)i * kColTileH + 8 * w, len, b);
-    split_cols_entries<NP, QT>(T, b, s, j0, (int64_t)i * kColTileH, S.nvec_pad, k_pad, S.planes, tile);
+    split_cols_entries<NP, QT>(T, b, s, j0, (int64_t)i * kColTileH, S.nvec, S.nvec_pad, k_pad, S.planes, tile);
     if (i >= kStripCtas) __syncthreads();            // the tile is read before the next one is staged
   }
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");     // no block leaves while its maxima may be read
@@ -771,8 +774,8 @@ __global__ void __launch_bounds__(256, KIND == kSideAny && NP > 5 ? 2 : 3) split
     colmax_side(S, l, len);
   else if (kind == kSideWarp)
     split_row_warp<true, NP, QT>(T, l * 8 + (threadIdx.x >> 5), S.nvec, len, S.X, S.ld, S.nvec_pad, k_pad, S.shifts,
-                                 S.planes, nullptr, false, true);
-  else
+                                 S.planes, nullptr, false, false, true);
+  else if (l < S.nvec)
     split_row<true, NP, QT>(T, l, S.nvec, len, S.X, S.ld, S.nvec_pad, k_pad, S.shifts, S.planes, nullptr, false, true);
 }
 
@@ -786,7 +789,7 @@ __global__ void __launch_bounds__(256, NP > 5 ? 2 : 3) split_tiles_kernel(const 
   const bool second = (int)blockIdx.x < b.blocks2;
   const SplitSide& S = second ? b : a;
   const int l = second ? blockIdx.x : (int)blockIdx.x - b.blocks2;
-  const int nbx = (int)(S.nvec_pad / kColTileJ);
+  const int nbx = (int)((S.nvec + kColTileJ - 1) / kColTileJ);
   const int64_t j0 = (int64_t)(l % nbx) * kColTileJ, hbase = (int64_t)(l / nbx) * kColTileH;
   const int64_t j = j0 + (threadIdx.x & 31);
   const bool live = j < S.nvec;
@@ -797,7 +800,8 @@ __global__ void __launch_bounds__(256, NP > 5 ? 2 : 3) split_tiles_kernel(const 
   const uint64_t m = live ? ld_dep(S.colmax + j) : 0ull;
   const int32_t s = shift_from_maxbits(m >> 63 ? 0ull : m, T.bits);
   if (hbase == 0 && live && threadIdx.x < 32) S.shifts[j] = s + (m >> 63 ? kBadMark : 0);
-  split_cols_entries<NP, QT>(T, v, s, j0, hbase, S.nvec_pad, k_pad, S.planes, reinterpret_cast<uint32_t*>(col_tile));
+  split_cols_entries<NP, QT>(T, v, s, j0, hbase, S.nvec, S.nvec_pad, k_pad, S.planes,
+                             reinterpret_cast<uint32_t*>(col_tile));
 }
 
 // Transpose of a rows x cols block of doubles (row pitch ld) into cols x rows
@@ -835,13 +839,14 @@ int pieces_for(int bits) { return bits <= 61 ? 4 : bits <= 64 ? 5 : 7; }
 
 template <bool kBF16, int NP, int QT>
 void split_rows_qt(const OzTables& t, int64_t nvec, int64_t len, const double* X, int64_t ld, int64_t nvec_pad,
-                   int64_t k_pad, int32_t* shifts, void* planes, int32_t* flag, cudaStream_t st, bool given) {
+                   int64_t k_pad, int32_t* shifts, void* planes, int32_t* flag, cudaStream_t st, bool given,
+                   bool pad) {
+  const int64_t rows = pad ? nvec_pad : nvec;
   if (k_pad <= 1024)                             // short rows: one warp per row
-    split_rows_warp_kernel<kBF16, NP, QT><<<(unsigned)(nvec_pad / 8), 256, 0, st>>>(t, nvec, len, X, ld, nvec_pad,
-                                                                                     k_pad, shifts, planes, flag,
-                                                                                     given);
+    split_rows_warp_kernel<kBF16, NP, QT><<<(unsigned)((rows + 7) / 8), 256, 0, st>>>(
+        t, nvec, len, X, ld, nvec_pad, k_pad, shifts, planes, flag, given, pad);
   else
-    split_rows_kernel<kBF16, NP, QT><<<(unsigned)nvec_pad, 256, 0, st>>>(t, nvec, len, X, ld, nvec_pad, k_pad, shifts,
+    split_rows_kernel<kBF16, NP, QT><<<(unsigned)rows, 256, 0, st>>>(t, nvec, len, X, ld, nvec_pad, k_pad, shifts,
                                                                           planes, flag, given);
 }
 
@@ -849,33 +854,36 @@ void split_rows_qt(const OzTables& t, int64_t nvec, int64_t len, const double* X
 // compile time; other counts read it from the table
 template <bool kBF16, int NP>
 void split_rows_np(const OzTables& t, int64_t nvec, int64_t len, const double* X, int64_t ld, int64_t nvec_pad,
-                   int64_t k_pad, int32_t* shifts, void* planes, int32_t* flag, cudaStream_t st, bool given) {
+                   int64_t k_pad, int32_t* shifts, void* planes, int32_t* flag, cudaStream_t st, bool given,
+                   bool pad) {
   if (t.Q == 16)
-    split_rows_qt<kBF16, NP, 16>(t, nvec, len, X, ld, nvec_pad, k_pad, shifts, planes, flag, st, given);
+    split_rows_qt<kBF16, NP, 16>(t, nvec, len, X, ld, nvec_pad, k_pad, shifts, planes, flag, st, given, pad);
   else
-    split_rows_qt<kBF16, NP, 0>(t, nvec, len, X, ld, nvec_pad, k_pad, shifts, planes, flag, st, given);
+    split_rows_qt<kBF16, NP, 0>(t, nvec, len, X, ld, nvec_pad, k_pad, shifts, planes, flag, st, given, pad);
 }
 
 template <int NP, int QT>
 cudaError_t split_cols_bf16_qt(const OzTables& t, int64_t nvec, int64_t len, const double* X, int64_t ld,
-                               int64_t nvec_pad, int64_t k_pad, const int32_t* shifts, void* planes, cudaStream_t st) {
+                               int64_t nvec_pad, int64_t k_pad, const int32_t* shifts, void* planes, cudaStream_t st,
+                               bool pad) {
+  const int64_t nstore = pad ? nvec_pad : nvec;
   const int smem = (QT > 0 ? QT : t.Q) * kColPlaneWords * 4;
   cudaError_t e = cudaFuncSetAttribute(split_cols_bf16_kernel<NP, QT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (QT > 0 ? QT : OZ_MAX_MODULI) * kColPlaneWords * 4);
   if (e != cudaSuccess) return e;
-  dim3 g((unsigned)(nvec_pad / kColTileJ), (unsigned)(k_pad / kColTileH));
-  split_cols_bf16_kernel<NP, QT><<<g, 256, smem, st>>>(t, nvec, len, X, ld, nvec_pad, k_pad, shifts,
+  dim3 g((unsigned)((nstore + kColTileJ - 1) / kColTileJ), (unsigned)(k_pad / kColTileH));
+  split_cols_bf16_kernel<NP, QT><<<g, 256, smem, st>>>(t, nvec, len, X, ld, nstore, nvec_pad, k_pad, shifts,
                                                        static_cast<uint16_t*>(planes));
   return cudaGetLastError();
 }
 
 template <bool kBF16, int NP>
 cudaError_t split_cols_np(const OzTables& t, int64_t nvec, int64_t len, const double* X, int64_t ld, int64_t nvec_pad,
-                          int64_t k_pad, const int32_t* shifts, void* planes, cudaStream_t st) {
+                          int64_t k_pad, const int32_t* shifts, void* planes, cudaStream_t st, bool pad) {
   if constexpr (kBF16) {
     if constexpr (NP <= 5)
-      if (t.Q == 16) return split_cols_bf16_qt<NP, 16>(t, nvec, len, X, ld, nvec_pad, k_pad, shifts, planes, st);
-    return split_cols_bf16_qt<NP, 0>(t, nvec, len, X, ld, nvec_pad, k_pad, shifts, planes, st);
+      if (t.Q == 16) return split_cols_bf16_qt<NP, 16>(t, nvec, len, X, ld, nvec_pad, k_pad, shifts, planes, st, pad);
+    return split_cols_bf16_qt<NP, 0>(t, nvec, len, X, ld, nvec_pad, k_pad, shifts, planes, st, pad);
   } else {
     dim3 g((unsigned)(nvec_pad / 64), (unsigned)(k_pad / 64));
     split_cols_kernel<kBF16, NP><<<g, 256, 0, st>>>(t, nvec, len, X, ld, nvec_pad, k_pad, shifts, planes);
@@ -935,12 +943,12 @@ SplitSide split_side(const SplitOperand& o, int64_t len, int64_t k_pad) {
   s.kind = o.contiguous ? (k_pad <= 1024 ? kSideWarp : kSideRow) : k_pad <= kStripMaxK ? kSideStrip : kSideTile;
   s.blocks2 = 0;
   switch (s.kind) {
-    case kSideRow: s.blocks1 = (int)o.nvec_pad; break;
-    case kSideWarp: s.blocks1 = (int)(o.nvec_pad / 8); break;
-    case kSideStrip: s.blocks1 = (int)(o.nvec_pad / kColTileJ) * kStripCtas; break;
+    case kSideRow: s.blocks1 = (int)round_up(o.nvec, kStripCtas); break;
+    case kSideWarp: s.blocks1 = (int)round_up((o.nvec + 7) / 8, kStripCtas); break;
+    case kSideStrip: s.blocks1 = (int)((o.nvec + kColTileJ - 1) / kColTileJ) * kStripCtas; break;
     default:
       s.blocks1 = (int)((o.nvec + 31) / 32 * ((len + 255) / 256));
-      s.blocks2 = (int)(o.nvec_pad / kColTileJ * (k_pad / kColTileH));
+      s.blocks2 = (int)((o.nvec + kColTileJ - 1) / kColTileJ * (k_pad / kColTileH));
   }
   return s;
 }
@@ -968,15 +976,15 @@ cudaError_t launch_split_both(const OzTables& t, const SplitOperand& A, const Sp
 
 cudaError_t launch_split_rows(const OzTables& t, int64_t nvec, int64_t len, const double* X, int64_t ld,
                               int64_t nvec_pad, int64_t k_pad, int32_t* shifts, void* planes, int bf16,
-                              int32_t* flag, cudaStream_t st, bool given) {
-  if (nvec_pad == 0) return cudaSuccess;
+                              int32_t* flag, cudaStream_t st, bool given, bool pad) {
+  if (nvec_pad == 0 || (nvec == 0 && !pad)) return cudaSuccess;
   switch (pieces_for(t.bits) * 2 + (bf16 ? 1 : 0)) {
-    case 9: split_rows_np<true, 4>(t, nvec, len, X, ld, nvec_pad, k_pad, shifts, planes, flag, st, given); break;
-    case 8: split_rows_np<false, 4>(t, nvec, len, X, ld, nvec_pad, k_pad, shifts, planes, flag, st, given); break;
-    case 11: split_rows_np<true, 5>(t, nvec, len, X, ld, nvec_pad, k_pad, shifts, planes, flag, st, given); break;
-    case 10: split_rows_np<false, 5>(t, nvec, len, X, ld, nvec_pad, k_pad, shifts, planes, flag, st, given); break;
-    case 15: split_rows_np<true, 7>(t, nvec, len, X, ld, nvec_pad, k_pad, shifts, planes, flag, st, given); break;
-    default: split_rows_np<false, 7>(t, nvec, len, X, ld, nvec_pad, k_pad, shifts, planes, flag, st, given); break;
+    case 9: split_rows_np<true, 4>(t, nvec, len, X, ld, nvec_pad, k_pad, shifts, planes, flag, st, given, pad); break;
+    case 8: split_rows_np<false, 4>(t, nvec, len, X, ld, nvec_pad, k_pad, shifts, planes, flag, st, given, pad); break;
+    case 11: split_rows_np<true, 5>(t, nvec, len, X, ld, nvec_pad, k_pad, shifts, planes, flag, st, given, pad); break;
+    case 10: split_rows_np<false, 5>(t, nvec, len, X, ld, nvec_pad, k_pad, shifts, planes, flag, st, given, pad); break;
+    case 15: split_rows_np<true, 7>(t, nvec, len, X, ld, nvec_pad, k_pad, shifts, planes, flag, st, given, pad); break;
+    default: split_rows_np<false, 7>(t, nvec, len, X, ld, nvec_pad, k_pad, shifts, planes, flag, st, given, pad); break;
   }
   return cudaGetLastError();
 }
@@ -1011,19 +1019,19 @@ cudaError_t launch_shifts_rows(int bits, int64_t nvec, int64_t len, const double
 
 cudaError_t launch_split_cols(const OzTables& t, int64_t nvec, int64_t len, const double* X, int64_t ld,
                               int64_t nvec_pad, int64_t k_pad, int32_t* shifts, void* planes, int bf16,
-                              int32_t* flag, uint64_t* colmax, cudaStream_t st, bool given) {
-  if (nvec_pad == 0) return cudaSuccess;
+                              int32_t* flag, uint64_t* colmax, cudaStream_t st, bool given, bool pad) {
+  if (nvec_pad == 0 || (nvec == 0 && !pad)) return cudaSuccess;
   if (!given) {
     cudaError_t e0 = launch_shifts_cols(t.bits, nvec, len, X, ld, shifts, flag, colmax, st);
     if (e0 != cudaSuccess) return e0;
   }
   switch (pieces_for(t.bits) * 2 + (bf16 ? 1 : 0)) {
-    case 9: return split_cols_np<true, 4>(t, nvec, len, X, ld, nvec_pad, k_pad, shifts, planes, st);
-    case 8: return split_cols_np<false, 4>(t, nvec, len, X, ld, nvec_pad, k_pad, shifts, planes, st);
-    case 11: return split_cols_np<true, 5>(t, nvec, len, X, ld, nvec_pad, k_pad, shifts, planes, st);
-    case 10: return split_cols_np<false, 5>(t, nvec, len, X, ld, nvec_pad, k_pad, shifts, planes, st);
-    case 15: return split_cols_np<true, 7>(t, nvec, len, X, ld, nvec_pad, k_pad, shifts, planes, st);
-    default: return split_cols_np<false, 7>(t, nvec, len, X, ld, nvec_pad, k_pad, shifts, planes, st);
+    case 9: return split_cols_np<true, 4>(t, nvec, len, X, ld, nvec_pad, k_pad, shifts, planes, st, pad);
+    case 8: return split_cols_np<false, 4>(t, nvec, len, X, ld, nvec_pad, k_pad, shifts, planes, st, pad);
+    case 11: return split_cols_np<true, 5>(t, nvec, len, X, ld, nvec_pad, k_pad, shifts, planes, st, pad);
+    case 10: return split_cols_np<false, 5>(t, nvec, len, X, ld, nvec_pad, k_pad, shifts, planes, st, pad);
+    case 15: return split_cols_np<true, 7>(t, nvec, len, X, ld, nvec_pad, k_pad, shifts, planes, st, pad);
+    default: return split_cols_np<false, 7>(t, nvec, len, X, ld, nvec_pad, k_pad, shifts, planes, st, pad);
   }
 }
 
