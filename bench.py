@@ -648,7 +648,7 @@ def run_batch(args, rank, world, local):
         bg, label, tune = oz.autotune_batch(shapes, As, Bs, Cs)
         mode_desc = "autotuned: " + label
         launches = bg.launches() if isinstance(bg, oz.GroupedGemm) else \
-            sum(oz.launches_per_dgemm(False, False) for _ in shapes)
+            sum(oz.launches_per_dgemm(False, False, shape=sh) for sh in shapes)
     elif args.batch_mode == "grouped":
         bg = oz.GroupedGemm(As, Bs, Cs)
         bg.capture()
@@ -656,7 +656,7 @@ def run_batch(args, rank, world, local):
     else:
         bg, tune = oz.autotune_batched(shapes, As, Bs, Cs, candidates=(1, 2, 4, 8, 16))
         mode_desc = f"oz_dgemm_batched on {bg.nstreams} streams"
-        launches = sum(oz.launches_per_dgemm() for _ in shapes)
+        launches = sum(oz.launches_per_dgemm(shape=sh) for sh in shapes)
     for _ in range(max(args.warmup, 1)):
         bg.replay()
     torch.cuda.synchronize()

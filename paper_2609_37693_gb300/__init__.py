@@ -370,14 +370,32 @@ class PlanFP(Plan):
         return f"PlanFP(format={self.format}, q={self.q}, channels={self.channels}, bits={self.bits})"
 
 
+_torch = None
+
+
+def _import_torch():
+    global _torch
+    if _torch is None:
+        import torch
+        _torch = torch
+    return _torch
+
+
 def _stream_handle(stream=None):
-    import torch
+    torch = _import_torch()
     s = torch.cuda.current_stream() if stream is None else stream
     return ctypes.c_void_p(s.cuda_stream)
 
 
+def _raw_stream():
+    """The current stream of the current device as an integer handle, without
+    building a torch Stream object (3 us, a tenth of a small product)."""
+    torch = _import_torch()
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+
+
 def workspace(plan: Plan, m: int, n: int, k: int, device=None):
-    import torch
+    torch = _import_torch()
     nbytes = plan.workspace_bytes(m, n, k)
     return torch.empty(max(nbytes, 256), dtype=torch.uint8, device=device or "cuda")
 
@@ -385,38 +403,43 @@ def workspace(plan: Plan, m: int, n: int, k: int, device=None):
 def dgemm(A, B, plan: Plan | None = None, trans_a: bool = False, trans_b: bool = False, out=None, ws=None,
           stream=None):
     """C = op(A) op(B) for float64 CUDA tensors (row-major, unit inner stride)."""
-    import torch
-    if A.dtype != torch.float64 or B.dtype != torch.float64 or not A.is_cuda or not B.is_cuda:
-        raise TypeError("dgemm takes float64 CUDA tensors")
-    if A.dim() != 2 or B.dim() != 2 or (A.numel() and A.stride(1) != 1) or (B.numel() and B.stride(1) != 1):
-        raise ValueError("dgemm takes 2-D tensors with unit inner stride")
-    m, k = (A.shape[1], A.shape[0]) if trans_a else (A.shape[0], A.shape[1])
-    k2, n = (B.shape[1], B.shape[0]) if trans_b else (B.shape[0], B.shape[1])
-    if k != k2:
-        raise ValueError(f"inner dimensions differ: {k} vs {k2}")
+    m, n, k, lda, ldb = _operands(A, B, trans_a, trans_b, "dgemm")
     if plan is None:
         plan = Plan(16, 0, max(k, 1))
-    C = out if out is not None else torch.empty((m, n), dtype=torch.float64, device=A.device)
+    if out is None:
+        C, ldc = _torch.empty((m, n), dtype=A.dtype, device=A.device), max(n, 1)
+    else:
+        C, ldc = out, _ld(out)
     if ws is None:
         ws = workspace(plan, m, n, k, A.device)
-    st = oz_dgemm(plan.handle, int(trans_a), int(trans_b), m, n, k, A.data_ptr(), _ld(A),
-                  B.data_ptr(), _ld(B), C.data_ptr(), _ld(C), ws.data_ptr(),
-                  ws.numel(), _stream_handle(stream))
-    _check(st, "oz_dgemm")
+    st = _lib.oz_dgemm(plan.handle, 1 if trans_a else 0, 1 if trans_b else 0, m, n, k, A.data_ptr(), lda,
+                       B.data_ptr(), ldb, C.data_ptr(), ldc, ws.data_ptr(), ws.numel(),
+                       _raw_stream() if stream is None else stream.cuda_stream)
+    if st != OZ_OK:
+        raise OzError(st, "oz_dgemm")
     return C
 
 
 def _operands(A, B, trans_a, trans_b, what):
-    import torch
-    if A.dtype != torch.float64 or B.dtype != torch.float64 or not A.is_cuda or not B.is_cuda:
+    """(m, n, k, lda, ldb) of a product of float64 CUDA tensors, or an error.
+    Each tensor's shape and strides are read once: at 256 x 256 x 256 the calls
+    on tensors cost more than the launches."""
+    f64 = _import_torch().float64
+    if A.dtype != f64 or B.dtype != f64 or not A.is_cuda or not B.is_cuda:
         raise TypeError(f"{what} takes float64 CUDA tensors")
-    if A.dim() != 2 or B.dim() != 2 or (A.numel() and A.stride(1) != 1) or (B.numel() and B.stride(1) != 1):
+    sa, sb = A.shape, B.shape
+    if len(sa) != 2 or len(sb) != 2:
         raise ValueError(f"{what} takes 2-D tensors with unit inner stride")
-    m, k = (A.shape[1], A.shape[0]) if trans_a else (A.shape[0], A.shape[1])
-    k2, n = (B.shape[1], B.shape[0]) if trans_b else (B.shape[0], B.shape[1])
+    (ra, ca), (rb, cb) = sa, sb
+    ta, tb = A.stride(), B.stride()
+    if (ra and ca and ta[1] != 1) or (rb and cb and tb[1] != 1):
+        raise ValueError(f"{what} takes 2-D tensors with unit inner stride")
+    m, k = (ca, ra) if trans_a else (ra, ca)
+    k2, n = (cb, rb) if trans_b else (rb, cb)
     if k != k2:
         raise ValueError(f"inner dimensions differ: {k} vs {k2}")
-    return m, n, k
+    # as _ld
+    return m, n, k, max(ta[0] if ra and ca else ca, 1), max(tb[0] if rb and cb else cb, 1)
 
 
 def dgemm_blocked(A, B, plan: Plan, k_slab: int, trans_a: bool = False, trans_b: bool = False, out=None, ws=None,
@@ -425,25 +448,36 @@ def dgemm_blocked(A, B, plan: Plan, k_slab: int, trans_a: bool = False, trans_b:
     of k_slab terms, each slab's digits added into a running residue (the same
     bits as ``dgemm`` wherever both apply; K up to ``plan.k_rec``, slabs up to
     ``plan.k_acc``). The workspace holds one slab's planes."""
-    import torch
-    m, n, k = _operands(A, B, trans_a, trans_b, "dgemm_blocked")
+    torch = _import_torch()
+    m, n, k, lda, ldb = _operands(A, B, trans_a, trans_b, "dgemm_blocked")
     C = out if out is not None else torch.empty((m, n), dtype=torch.float64, device=A.device)
     if ws is None:
         nbytes = oz_blocked_workspace_bytes(plan.handle, m, n, max(min(int(k_slab), k), 1))
         ws = torch.empty(max(nbytes, 256), dtype=torch.uint8, device=A.device)
-    st = oz_dgemm_blocked(plan.handle, int(trans_a), int(trans_b), m, n, k, int(k_slab), A.data_ptr(), _ld(A),
-                          B.data_ptr(), _ld(B), C.data_ptr(), _ld(C), ws.data_ptr(), ws.numel(),
+    st = oz_dgemm_blocked(plan.handle, int(trans_a), int(trans_b), m, n, k, int(k_slab), A.data_ptr(), lda,
+                          B.data_ptr(), ldb, C.data_ptr(), _ld(C), ws.data_ptr(), ws.numel(),
                           _stream_handle(stream))
     _check(st, "oz_dgemm_blocked")
     return C
 
 
-def launches_per_dgemm(trans_a: bool = False, trans_b: bool = False, engine: int = OZ_ENGINE_TC) -> int:
-    """Kernels one INT8 oz_dgemm launches without a split of K: A's rows split
-    in one kernel (its columns, for trans_a, in three: column maxima, shifts,
-    split); B's columns in three (bf16 planes) or transposed and split as rows
-    (two, int8 planes of the IMMA engine); one when trans_b; then the GEMM and
-    the reconstruct."""
+def launches_per_dgemm(trans_a: bool = False, trans_b: bool = False, engine: int = OZ_ENGINE_TC, shape=None) -> int:
+    """Kernels one INT8 oz_dgemm launches without a split of K, the GEMM and
+    the reconstruct among them. Large products (shape None, or past the bounds
+    below) split A's rows in one kernel (its columns, for trans_a, in three:
+    column maxima, shifts, split) and B's columns in three (bf16 planes) or
+    transposed and split as rows (two, int8 planes of the IMMA engine); one when
+    trans_b. On the TC engines a shape (m, n, k) whose padded k is at most 1024,
+    or whose padded operands have at most 2^22 entries, splits both operands
+    together: one kernel, a second one when only the first bound holds and an
+    operand's vectors are columns, and one for the tiles of longer columns."""
+    if shape is not None and engine != OZ_ENGINE_IMMA:
+        m_pad, n_pad, k_pad = round_up(shape[0], 256), round_up(shape[1], 256), round_up(shape[2], 128)
+        columns = bool(trans_a) or not trans_b
+        if (m_pad + n_pad) * k_pad <= 1 << 22:
+            return 3 + (columns and k_pad > 1024)
+        if k_pad <= 1024:
+            return 3 + columns
     a = 3 if trans_a else 1
     b = 1 if trans_b else (2 if engine == OZ_ENGINE_IMMA else 3)
     return a + b + 2
@@ -474,11 +508,6 @@ def plan_for(k: int, q: int = 16, engine: int = OZ_ENGINE_AUTO) -> Plan:
 def _matmul_op(A, B, trans_a: bool, trans_b: bool, q: int, engine: int):
     k = A.shape[0] if trans_a else A.shape[1]
     return dgemm(A, B, plan_for(k, q, engine), trans_a=trans_a, trans_b=trans_b)
-
-
-def _import_torch():
-    import torch
-    return torch
 
 
 class EmuMatmul:
@@ -690,7 +719,7 @@ def autotune_blocked(A, B, candidates=None, bits: int = 53, reps: int = 2, strea
     blocked_candidates(K, bits) -- and return (label, plan, k_slab) of the
     fastest with {label: ms}."""
     torch = _import_torch()
-    m, n, k = _operands(A, B, False, False, "autotune_blocked")
+    m, n, k, _, _ = _operands(A, B, False, False, "autotune_blocked")
     cands = candidates if candidates is not None else blocked_candidates(k, bits)
     if not cands:
         raise OzError(OZ_ERR_K_TOO_LARGE, "autotune_blocked")
