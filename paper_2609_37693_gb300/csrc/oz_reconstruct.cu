@@ -556,11 +556,13 @@ __device__ __forceinline__ void multiple_of_P(const uint4* kP, int q, uint32_t (
 // round-to-nearest-even increment (a carry out of the significand bumps the
 // exponent field, up to infinity). Returns false (out unset) otherwise.
 template <int L>
-__device__ __forceinline__ bool round_groups_fast(const uint4* kP, const uint32_t (&s)[L], float f, int ex,
+__device__ __forceinline__ bool round_groups_fast(const uint4* kP, int kmax, const uint32_t (&s)[L], float f, int ex,
                                                   uint64_t& out) {
-  const float kf = rintf(f);                               // at most rg_multiples - 1: S / P is below it
+  const float kf = rintf(f);
   uint32_t m[L], y[L];
-  multiple_of_P<L>(kP, (int)kf, y);
+  // digits past n in a row's padding are whatever the workspace holds, and their
+  // quotient may lie past the table: kmax, its last multiple
+  multiple_of_P<L>(kP, min((int)kf, kmax), y);
 #pragma unroll
   for (int l = 0; l < L; ++l) m[l] = s[l];
   sub_limbs<L>(m, y);
@@ -678,7 +680,7 @@ __device__ __forceinline__ void rec4_groups(const OzTables& T, const uint4* kP, 
     uint32_t S[L];
     float f;
     crt_groups<NT, NP2, NQ4, L>(T, w, e, S, f);
-    if (!round_groups_fast<L>(kP, S, f, -(si + tj[e]), out[e])) slow |= 1u << e;
+    if (!round_groups_fast<L>(kP, rg_multiples(Q) - 1, S, f, -(si + tj[e]), out[e])) slow |= 1u << e;
   }
   if (slow) {                                              // rare: one branch for the four entries
 #pragma unroll
