@@ -99,6 +99,42 @@ static __device__ __forceinline__ uint64_t warp_max_u64(uint64_t v) {
   return v;
 }
 
+// The largest |x| bit pattern over row[h], h = t, t + step, ... (t < step),
+// and whether any of those entries is not finite: 16-byte loads (two
+// entries) when the row is 16-byte aligned, four of them in flight per
+// iteration, so that a short row's maximum is not a chain of load latencies.
+static __device__ __forceinline__ void row_absmax(const uint64_t* row, int64_t len, int t, int step,
+                                           uint64_t& mx, uint32_t& bad) {
+  auto fold = [&](uint64_t b) {
+    b &= kAbsMask;
+    bad |= (uint32_t)((b >> 52) == 0x7ff);
+    mx = b > mx ? b : mx;
+  };
+  if ((reinterpret_cast<uintptr_t>(row) & 15) == 0) {
+    const ulonglong2* r2 = reinterpret_cast<const ulonglong2*>(row);
+    const int64_t np = len >> 1;
+    int64_t p = t;
+    for (; p + 3 * (int64_t)step < np; p += 4 * (int64_t)step) {
+      ulonglong2 v[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) v[u] = ld_dep(r2 + p + u * step);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        fold(v[u].x);
+        fold(v[u].y);
+      }
+    }
+    for (; p < np; p += step) {
+      const ulonglong2 v = ld_dep(r2 + p);
+      fold(v.x);
+      fold(v.y);
+    }
+    if ((len & 1) && t == 0) fold(ld_dep(row + len - 1));
+  } else {
+    for (int64_t h = t; h < len; h += step) fold(ld_dep(row + h));
+  }
+}
+
 // (a + b) mod m in each byte, for bytes a, b in [0, m) and m < 256 given as
 // mm = m * 0x01010101: a - (m - b), plus m in the bytes where that borrows.
 // The GEMM epilogues of a blocked call add a slab's digits into the earlier

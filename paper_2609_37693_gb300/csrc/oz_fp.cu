@@ -272,6 +272,226 @@ __global__ void __launch_bounds__(256) split_fp_cols_kernel(const __grid_constan
   }
 }
 
+// ---------------------------------------------------------------------------
+// The same splits through a table in shared memory (plans of at most 55 bits
+// whose moduli are at most 1366: every beta = 53 configuration). The kernels
+// above are bound by their instructions and by the look-ups in L1: a 32-bit Barrett
+// reduction and a gather of up to 32 lines per entry and channel. Here the residue is
+// formed in exact fp32 as in oz_split.cu, two entries per packed operation:
+// |a'| in a 22-bit piece and three of 11 bits, y = P0 + sum P_i c_i with
+// |y| < 2^22 + 3 * 2047 * 683 < 2^23, r = y - m rint(y / m) in [-m/2, m/2] (a tie of
+// an even modulus falls to either end, both hold its class), and r + 1.5 2^23 is,
+// as bits, the index of the code word in the channel's table by balanced residue.
+// Blocks stay for many rows or tiles, since each copies the whole table (27 KB
+// for E4M3) into shared memory first.
+// ---------------------------------------------------------------------------
+struct Pieces11 {
+  float p[4];
+};
+
+__device__ __forceinline__ Pieces11 pieces11(uint64_t bits, int32_t s) {
+  if (((bits >> 52) & 0x7ff) == 0x7ff) bits = 0;         // non-finite: flagged with the maxima
+  const Trunc t = truncate(bits, s);
+  const float sg = t.neg ? -1.0f : 1.0f;
+  const float off = t.neg ? 8388608.0f : -8388608.0f;
+  Pieces11 P;
+  P.p[0] = fmaf(__int_as_float(0x4B000000u | ((uint32_t)t.mag & 0x3fffffu)), sg, off);      // +-v, exact
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+    P.p[i + 1] = fmaf(__int_as_float(0x4B000000u | ((uint32_t)(t.mag >> (22 + 11 * i)) & 0x7ffu)), sg, off);
+  return P;
+}
+
+// The code words of eight entries in channel c; tab: the table's shared address.
+__device__ __forceinline__ void table_words(const OzFpTables& F, int c, uint32_t tab, const Pieces11 (&P)[8],
+                                            uint32_t (&w)[8]) {
+  const float2 kC = make_float2(12582912.0f, 12582912.0f), kCn = make_float2(-12582912.0f, -12582912.0f);
+  const float2 inv = make_float2(F.invm[c], F.invm[c]), nm = make_float2(-F.mf[c], -F.mf[c]);
+  const float2 c0 = make_float2(F.c11f[0][c], F.c11f[0][c]), c1 = make_float2(F.c11f[1][c], F.c11f[1][c]),
+               c2 = make_float2(F.c11f[2][c], F.c11f[2][c]);
+  const uint32_t base = tab + 4u * (F.ch_coff[c] - 0x4B400000u);     // word of residue 0, less 4 * bits(1.5 * 2^23)
+#pragma unroll
+  for (int e = 0; e < 8; e += 2) {
+    float2 y = make_float2(P[e].p[0], P[e + 1].p[0]);
+    y = __ffma2_rn(make_float2(P[e].p[1], P[e + 1].p[1]), c0, y);
+    y = __ffma2_rn(make_float2(P[e].p[2], P[e + 1].p[2]), c1, y);
+    y = __ffma2_rn(make_float2(P[e].p[3], P[e + 1].p[3]), c2, y);
+    const float2 q = __fadd2_rn(__ffma2_rn(y, inv, kC), kCn);
+    const float2 r = __fadd2_rn(__ffma2_rn(q, nm, y), kC);
+    asm("ld.shared.u32 %0, [%1];" : "=r"(w[e]) : "r"(base + 4u * __float_as_uint(r.x)));
+    asm("ld.shared.u32 %0, [%1];" : "=r"(w[e + 1]) : "r"(base + 4u * __float_as_uint(r.y)));
+  }
+}
+
+__device__ __forceinline__ uint32_t load_code_table(const OzFpTables& F, uint32_t* sm) {
+  for (int i = threadIdx.x; i < F.cw_total; i += (int)blockDim.x) sm[i] = __ldg(F.cwords + i);
+  __syncthreads();
+  return smem_u32(sm);
+}
+
+template <int CB>
+__global__ void __launch_bounds__(256, 3) split_fp_rows_tab_kernel(const __grid_constant__ OzFpTables F, int bits,
+                                                                   int64_t nvec, int64_t len,
+                                                                   const double* __restrict__ X, int64_t ld,
+                                                                   int64_t nvec_pad, int64_t k_pad,
+                                                                   int32_t* __restrict__ shifts,
+                                                                   uint8_t* __restrict__ planes,
+                                                                   int32_t* __restrict__ flag, bool given) {
+  extern __shared__ uint32_t code_tab[];
+  __shared__ uint64_t red[8];
+  __shared__ int32_t s_sh;
+  const uint32_t tab = load_code_table(F, code_tab);
+  const int tid = threadIdx.x;
+  const int64_t row_bytes = CB == 4 ? k_pad / 2 : k_pad;
+  const int64_t plane = nvec_pad * row_bytes;
+  for (int64_t v = blockIdx.x; v < nvec_pad; v += gridDim.x) {
+    const bool live = v < nvec;
+    const uint64_t* row = reinterpret_cast<const uint64_t*>(X) + (live ? v * ld : 0);
+    int32_t s;
+    if (given) {                      // the shift of the whole row is known (blocked call)
+      s = live ? shifts[v] : 0;
+    } else {
+      uint64_t mx = 0;
+      uint32_t bad = 0;
+      if (live) row_absmax(row, len, tid, 256, mx, bad);
+      mx = warp_max_u64(mx);
+      bad = __any_sync(0xffffffffu, bad);
+      if ((tid & 31) == 0) red[tid >> 5] = mx | (bad ? (1ull << 63) : 0);
+      __syncthreads();
+      if (tid == 0) {
+        uint64_t m = 0, anybad = 0;
+        for (int w = 0; w < 8; ++w) {
+          anybad |= red[w] >> 63;
+          const uint64_t x = red[w] & kAbsMask;
+          m = x > m ? x : m;
+        }
+        if (anybad && flag) atomicOr(flag, 1);
+        const int32_t s0 = live ? shift_from_maxbits(anybad ? 0 : m, bits) : 0;
+        s_sh = s0;
+        if (live) shifts[v] = s0;
+      }
+      __syncthreads();                // s_sh is rewritten after the next row's first barrier only
+      s = s_sh;
+    }
+    uint8_t* out_row = planes + v * row_bytes;
+    const bool vec = live && ((reinterpret_cast<uintptr_t>(row) & 15) == 0);
+    // every thread runs every pass (the shuffle of the 6-bit path needs both lanes)
+    for (int64_t base = 0; base < k_pad; base += 256 * 8) {
+      const int64_t h0 = base + (int64_t)tid * 8;
+      const bool active = h0 < k_pad;
+      uint64_t b[8];
+      if (vec && h0 + 8 <= len) {
+#pragma unroll
+        for (int e = 0; e < 8; e += 2) {
+          const ulonglong2 w = __ldg(reinterpret_cast<const ulonglong2*>(row + h0 + e));
+          b[e] = w.x;
+          b[e + 1] = w.y;
+        }
+      } else {
+#pragma unroll
+        for (int e = 0; e < 8; ++e) b[e] = (live && h0 + e < len) ? __ldg(row + h0 + e) : 0ull;
+      }
+      Pieces11 P[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) P[e] = pieces11(b[e], s);
+      for (int c = 0; c < F.nch; ++c) {
+        uint32_t w[8];
+        table_words(F, c, tab, P, w);
+        const int p0 = F.ch_plane0[c], np = F.ch_nplanes[c];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+          if (q >= np) break;
+          uint8_t* dst = out_row + (int64_t)(p0 + q) * plane;
+          const uint64_t pb = plane_bits8<CB>(w, q);
+          if constexpr (CB == 8) {
+            if (active) *reinterpret_cast<uint2*>(dst + h0) = make_uint2((uint32_t)pb, (uint32_t)(pb >> 32));
+          } else if constexpr (CB == 4) {
+            if (active) *reinterpret_cast<uint32_t*>(dst + h0 / 2) = (uint32_t)pb;
+          } else {
+            const uint64_t other = __shfl_xor_sync(0xffffffffu, pb, 1);
+            if (active && (tid & 1) == 0) *reinterpret_cast<uint4*>(dst + h0) = chunk6(pb, other);
+          }
+        }
+      }
+    }
+  }
+}
+
+// Strided vectors: tiles of 32 vectors x 128 entries, vectors fastest. Lane l holds
+// vector j0 + l and warp w its entries hbase + 8 w .. + 7 (each load reads 32
+// consecutive doubles of a row of X). A channel's planes are staged in shared
+// memory, rows of 128 (4-bit codes: 64) bytes at a pitch of 16 more, two buffers in
+// turn with one barrier per channel, and leave as whole rows: stored straight
+// from the lanes that hold them they went out in pieces of 32 or 16 bytes, which
+// bound the kernel (E2M1 494 us at 4096^2).
+constexpr int kFpTableMax = 48 * 1024;                                   // bytes of a plan's code table
+constexpr int kFpColThreads = 512, kFpColTileH = 128;
+constexpr int kFpStagePitch = 144, kFpStagePlane = 32 * kFpStagePitch;   // bytes
+
+template <int CB>
+__global__ void __launch_bounds__(kFpColThreads, 2) split_fp_cols_tab_kernel(const __grid_constant__ OzFpTables F,
+                                                                             int64_t nvec, int64_t len,
+                                                                             const double* __restrict__ X, int64_t ld,
+                                                                             int64_t nvec_pad, int64_t k_pad,
+                                                                             const int32_t* __restrict__ shifts,
+                                                                             uint8_t* __restrict__ planes) {
+  constexpr int kRow = CB == 4 ? kFpColTileH / 2 : kFpColTileH;          // bytes of a tile's plane row
+  constexpr int kRuns = kRow / 16, kPlaneRuns = 32 * kRuns;
+  extern __shared__ uint4 fp_smem[];                                     // [2][3] staged planes, then the table
+  uint8_t* const stage = reinterpret_cast<uint8_t*>(fp_smem);
+  uint32_t* const code_tab = reinterpret_cast<uint32_t*>(stage + 6 * kFpStagePlane);
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const uint32_t tab = load_code_table(F, code_tab);
+  const int64_t row_bytes = CB == 4 ? k_pad / 2 : k_pad;
+  const int64_t plane = nvec_pad * row_bytes;
+  const uint64_t* Xb = reinterpret_cast<const uint64_t*>(X);
+  const int64_t nbx = nvec_pad / 32, total = nbx * (k_pad / kFpColTileH);
+  uint32_t turn = 0;
+  for (int64_t t = blockIdx.x; t < total; t += gridDim.x) {
+    const int64_t j0 = (t % nbx) * 32, hbase = (t / nbx) * kFpColTileH;
+    const int64_t j = j0 + lane, h0 = hbase + 8 * w;
+    const bool live = j < nvec;
+    const int32_t s = live ? __ldg(shifts + j) : 0;
+    uint64_t b[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) b[e] = (live && h0 + e < len) ? __ldg(Xb + (h0 + e) * ld + j) : 0ull;
+    Pieces11 P[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) P[e] = pieces11(b[e], s);
+    uint8_t* const out = planes + j0 * row_bytes + (CB == 4 ? hbase / 2 : hbase);
+    for (int c = 0; c < F.nch; ++c, turn ^= 1u) {
+      uint32_t wd[8];
+      table_words(F, c, tab, P, wd);
+      const int p0 = F.ch_plane0[c], np = F.ch_nplanes[c];
+      uint8_t* const buf = stage + turn * 3 * kFpStagePlane;
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        if (q >= np) break;
+        const uint64_t pb = plane_bits8<CB>(wd, q);
+        uint8_t* const row = buf + q * kFpStagePlane + lane * kFpStagePitch;
+        if constexpr (CB == 8) {
+          *reinterpret_cast<uint2*>(row + 8 * w) = make_uint2((uint32_t)pb, (uint32_t)(pb >> 32));
+        } else if constexpr (CB == 4) {
+          *reinterpret_cast<uint32_t*>(row + 4 * w) = (uint32_t)pb;
+        } else {                                     // half of a 16-entry chunk: 6 of its 12 bytes, 2 of its 4 zeros
+          uint16_t* const d = reinterpret_cast<uint16_t*>(row + 16 * (w >> 1) + 6 * (w & 1));
+          d[0] = (uint16_t)pb;
+          d[1] = (uint16_t)(pb >> 16);
+          d[2] = (uint16_t)(pb >> 32);
+          *reinterpret_cast<uint16_t*>(row + 16 * (w >> 1) + 12 + 2 * (w & 1)) = 0;
+        }
+      }
+      __syncthreads();
+      // the other buffer was read before this barrier by every thread
+      for (int i = tid; i < np * kPlaneRuns; i += kFpColThreads) {
+        const int q = i / kPlaneRuns, r = i % kPlaneRuns / kRuns, ch = i % kRuns;
+        *reinterpret_cast<uint4*>(out + (int64_t)(p0 + q) * plane + r * row_bytes + 16 * ch) =
+            *reinterpret_cast<const uint4*>(buf + q * kFpStagePlane + r * kFpStagePitch + 16 * ch);
+      }
+    }
+  }
+}
+
 // =========================================================================
 // GEMMs + epilogue (tcgen05, kind::f8f6f4)
 // =========================================================================
@@ -1080,11 +1300,42 @@ cudaError_t split_fp_w(const OzTables& t, const OzFpTables& f, int contiguous, i
   return cudaGetLastError();
 }
 
+template <int CB>
+cudaError_t split_fp_tab(const OzTables& t, const OzFpTables& f, int contiguous, int64_t nvec, int64_t len,
+                         const double* X, int64_t ld, int64_t nvec_pad, int64_t k_pad, int32_t* shifts,
+                         uint8_t* planes, int32_t* flag, uint64_t* colmax, cudaStream_t st, bool given) {
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  if (contiguous) {
+    const int64_t most = 3 * (int64_t)sms;
+    split_fp_rows_tab_kernel<CB><<<(unsigned)(nvec_pad < most ? nvec_pad : most), 256, f.cw_total * 4, st>>>(
+        f, t.bits, nvec, len, X, ld, nvec_pad, k_pad, shifts, planes, flag, given);
+    return cudaGetLastError();
+  }
+  if (!given) {
+    e = launch_shifts_cols(t.bits, nvec, len, X, ld, shifts, flag, colmax, st);
+    if (e != cudaSuccess) return e;
+  }
+  const int smem = 6 * kFpStagePlane + f.cw_total * 4;
+  e = cudaFuncSetAttribute(split_fp_cols_tab_kernel<CB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           6 * kFpStagePlane + kFpTableMax);
+  if (e != cudaSuccess) return e;
+  const int64_t tiles = nvec_pad / 32 * (k_pad / kFpColTileH), most = 2 * (int64_t)sms;
+  split_fp_cols_tab_kernel<CB><<<(unsigned)(tiles < most ? tiles : most), kFpColThreads, smem, st>>>(
+      f, nvec, len, X, ld, nvec_pad, k_pad, shifts, planes);
+  return cudaGetLastError();
+}
+
 // beta > 64: |a'| in 128 bits and a fifth 16-bit piece
 template <int CB>
 cudaError_t split_fp(const OzTables& t, const OzFpTables& f, int contiguous, int64_t nvec, int64_t len,
                      const double* X, int64_t ld, int64_t nvec_pad, int64_t k_pad, int32_t* shifts, uint8_t* planes,
                      int32_t* flag, uint64_t* colmax, cudaStream_t st, bool given) {
+  if (f.split_tab && f.cw_total * 4 <= kFpTableMax)
+    return split_fp_tab<CB>(t, f, contiguous, nvec, len, X, ld, nvec_pad, k_pad, shifts, planes, flag, colmax, st,
+                            given);
   if (t.bits > 64)
     return split_fp_w<CB, true>(t, f, contiguous, nvec, len, X, ld, nvec_pad, k_pad, shifts, planes, flag, colmax,
                                 st, given);
@@ -1203,6 +1454,8 @@ cudaError_t launch_reconstruct16(const OzTables& T, int64_t m, int64_t n, const 
   if (m == 0 || n == 0) return cudaSuccess;
   if (ldy < n) return cudaErrorInvalidValue;
   if (T.limbs > 4) return launch_reconstruct16_wide(T, m, n, Y, ldy, s, t, C, ldc, st);   // widened budgets
+  const cudaError_t g = launch_reconstruct16_groups(T, m, n, Y, ldy, s, t, C, ldc, st);
+  if (g != cudaErrorNotSupported) return g;
   switch (T.npairs) {
     case 5: return launch16<5>(T, m, n, Y, ldy, s, t, C, ldc, st);
     case 6: return launch16<6>(T, m, n, Y, ldy, s, t, C, ldc, st);

@@ -50,6 +50,12 @@ struct OzTables {
   uint32_t rg_m2a[OZ_RG_MAX], rg_m2b[OZ_RG_MAX]; // quad: the products of its two pairs
   uint32_t rg_N[OZ_RG_MAX][5];                   // N_g = P / M_g, 32-bit limbs
   float rg_invM[OZ_RG_MAX];                      // 1 / M_g rounded to fp32 (S / P = sum_g t_g / M_g)
+  // The same for 16-bit digits (float formats, P < 2^125): rh_ng groups of
+  // consecutive moduli, group g the moduli rh_start[g] .. rh_start[g + 1] - 1 with
+  // weights rh_w[q] = M_g / m_q. rh_ng = 0: not available.
+  int rh_ng, rh_start[OZ_RG_MAX + 1];
+  uint32_t rh_w[OZ_TABLE_CAP], rh_N[OZ_RG_MAX][4];
+  float rh_invM[OZ_RG_MAX];
 };
 
 // A low-precision float configuration (Sec. "Forms and Channels"): channels
@@ -83,6 +89,14 @@ struct OzFpTables {
   // (m - i) mod m (the class of -x when x has class i); byte q of a word is
   // the code of the channel's plane q
   const uint32_t* words;
+  // The same words by balanced residue, for the split through shared memory:
+  // channel c's word of the class of r, |r| <= floor(m / 2), is
+  // cwords[ch_coff[c] + r]; cw_total words in all. c11f[i][c]: 2^(22 + 11 i) mod m
+  // nearest zero. split_tab: the bounds of that split hold (oz_fp.cu).
+  const uint32_t* cwords;
+  uint32_t ch_coff[OZ_TABLE_CAP];
+  int cw_total, split_tab;
+  float c11f[3][OZ_TABLE_CAP];
 };
 
 struct oz_plan_s {
@@ -294,6 +308,10 @@ cudaError_t launch_gemm_fp(const OzFpTables& f, int64_t m, int64_t n, int64_t m_
                            cudaStream_t st);
 cudaError_t launch_reconstruct16(const OzTables& t, int64_t m, int64_t n, const uint16_t* Y, int64_t ldy,
                                  const int32_t* s, const int32_t* tt, double* C, int64_t ldc, cudaStream_t st);
+// the same by groups of moduli (oz_reconstruct.cu): cudaErrorNotSupported when the
+// plan's tables or Y's pitch and base (multiples of 4 digits) do not serve it
+cudaError_t launch_reconstruct16_groups(const OzTables& t, int64_t m, int64_t n, const uint16_t* Y, int64_t ldy,
+                                        const int32_t* s, const int32_t* tt, double* C, int64_t ldc, cudaStream_t st);
 // shared by the split kernels: shifts of strided vectors (colmax must be zeroed)
 cudaError_t launch_shifts_cols(int bits, int64_t nvec, int64_t len, const double* X, int64_t ld, int32_t* shifts,
                                int32_t* flag, uint64_t* colmax, cudaStream_t st);

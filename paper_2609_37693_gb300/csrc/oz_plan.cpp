@@ -199,6 +199,42 @@ void fill_group_tables(OzTables* tp, const uint32_t* moduli, int Q, const Big& P
   t.rg_nq4 = nq4;
 }
 
+// Groups of consecutive moduli for the reconstruct of 16-bit digits: each group
+// takes moduli while its largest sum, (size) M_g, stays below 2^32. Left unset
+// unless the sum of these over the groups stays below 2^32 (each 64-bit limb
+// accumulator then holds), P is below 2^125 and the kernel's table of 32
+// multiples of P covers the sum (below Q P).
+void fill_digit16_groups(OzTables* tp, const uint32_t* moduli, int Q, const Big& P) {
+  OzTables& t = *tp;
+  t.rh_ng = 0;
+  if (Q < 2 || Q > 31 || P.bitlen() > 125) return;
+  int ng = 0, q = 0;
+  double tsum = 0.0;
+  while (q < Q) {
+    if (ng == OZ_RG_MAX) return;
+    uint64_t M = 1;
+    int e = q;
+    while (e < Q && (double)(e - q + 1) * (double)M * moduli[e] < 1073741824.0) M *= moduli[e++];
+    if (e == q) return;
+    t.rh_start[ng] = q;
+    for (int i = q; i < e; ++i) t.rh_w[i] = (uint32_t)(M / moduli[i]);
+    Big N = P;
+    for (int i = q; i < e; ++i) {
+      Big N2;
+      N.divmod(moduli[i], &N2);
+      N = N2;
+    }
+    for (int l = 0; l < 4; ++l) t.rh_N[ng][l] = N.w[l];
+    t.rh_invM[ng] = (float)(1.0 / (double)M);
+    tsum += (double)(e - q) * (double)M;
+    q = e;
+    ++ng;
+  }
+  if (tsum >= 4294967296.0) return;
+  t.rh_start[ng] = Q;
+  t.rh_ng = ng;
+}
+
 // Per-modulus constants and the CRT sum's limbs for moduli m[0..Q-1] (pairwise
 // coprime, each below 2^12): Barrett and reduction constants for the split
 // kernels, (P/m)^-1 mod m for the epilogue, and P, P/m, and the pair products
@@ -244,6 +280,7 @@ bool fill_crt_tables(OzTables* tp, const uint32_t* moduli, int Q, int bits) {
     for (int i = 0; i < OZ_MAX_LIMBS; ++i) t.Np[pi][i] = Np.w[i];
   }
   fill_group_tables(&t, moduli, Q, P);
+  fill_digit16_groups(&t, moduli, Q, P);
   return true;
 }
 

@@ -372,6 +372,20 @@ extern "C" oz_status oz_plan_create_fp(oz_plan* out, int format, int64_t k_hint,
       words.push_back(w);
     }
   }
+  // the same words by balanced residue r = -floor(m/2) .. floor(m/2) (an even m has
+  // its class m/2 at both ends), after them in the device table
+  const size_t centred = words.size();
+  f.split_tab = p->bits <= 55;               // pieces of 22 + 3 * 11 bits
+  for (int c = 0; c < cfg->nch; ++c) {
+    const int m = (int)f.m[c], h = m / 2;
+    f.ch_coff[c] = (uint32_t)(words.size() - centred) + (uint32_t)h;
+    for (int r = -h; r <= h; ++r) words.push_back(words[f.ch_woff[c] + (uint32_t)(r >= 0 ? r : m + r)]);
+    int64_t x = (1ll << 22) % m;
+    for (int i = 0; i < 3; ++i, x = (x << 11) % m) f.c11f[i][c] = (float)(x > h ? x - m : x);
+    // |y| < 2^22 + 3 (2^11 - 1) floor(m / 2) has to stay below 2^23
+    if ((1ll << 22) + 3ll * 2047 * h >= (1ll << 23)) f.split_tab = 0;
+  }
+  f.cw_total = (int)(words.size() - centred);
   // Without a CUDA device the plan still describes the configuration
   // (oz_plan_info_fp); products on it then return OZ_ERR_CUDA.
   int ndev = 0;
@@ -387,6 +401,7 @@ extern "C" oz_status oz_plan_create_fp(oz_plan* out, int format, int64_t k_hint,
     cudaGetLastError();
   }
   f.words = p->d_words;
+  f.cwords = p->d_words ? p->d_words + centred : nullptr;
   *out = p;
   return OZ_OK;
 }

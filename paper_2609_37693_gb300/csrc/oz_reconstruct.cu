@@ -598,21 +598,10 @@ __device__ __forceinline__ bool round_groups_fast(const uint4* kP, int kmax, con
   return true;
 }
 
-// Every other case, recomputed from the digits (wsm[q * QS], this thread's
-// shared-memory slots): the CRT sum S exactly (S < kmax P < 2^(32 L)),
-// X = S - qP corrected exactly into [-P/2, P/2), and the general rounding.
-template <int NT, int NP2, int NQ4, int QS>
-__device__ __noinline__ uint64_t round_groups_slow(const OzTables& T, const uint4* kP, const uint32_t* wsm, int e,
-                                                   int ex) {
-  constexpr int Q = 3 * NT + 2 * NP2 + 4 * NQ4, L = rg_limbs(Q);
-  uint32_t w[Q];
-#pragma unroll
-  for (int q = 0; q < Q; ++q) w[q] = wsm[q * QS];
-  uint32_t s[L], y[L];
-  float f;
-  crt_groups<NT, NP2, NQ4, L>(T, w, e, s, f);
-  multiple_of_P<L>(kP, min((int)rintf(f), rg_multiples(Q) - 1), y);
-  sub_limbs<L>(s, y);
+// fl(X 2^ex) of the candidate X in s (two's complement, |X| < 3P/2), corrected
+// exactly into [-P/2, P/2), by the general rounding.
+template <int L>
+__device__ __forceinline__ uint64_t round_exact(const OzTables& T, const uint32_t (&s)[L], int ex) {
   Limbs<L> X;
 #pragma unroll
   for (int l = 0; l < L; ++l) X.w[l] = s[l];
@@ -629,6 +618,24 @@ __device__ __noinline__ uint64_t round_groups_slow(const OzTables& T, const uint
     }
   }
   return round_to_binary64(X, neg, ex);
+}
+
+// Every other case, recomputed from the digits (wsm[q * QS], this thread's
+// shared-memory slots): the CRT sum S exactly (S < kmax P < 2^(32 L)),
+// X = S - qP corrected exactly into [-P/2, P/2), and the general rounding.
+template <int NT, int NP2, int NQ4, int QS>
+__device__ __noinline__ uint64_t round_groups_slow(const OzTables& T, const uint4* kP, const uint32_t* wsm, int e,
+                                                   int ex) {
+  constexpr int Q = 3 * NT + 2 * NP2 + 4 * NQ4, L = rg_limbs(Q);
+  uint32_t w[Q];
+#pragma unroll
+  for (int q = 0; q < Q; ++q) w[q] = wsm[q * QS];
+  uint32_t s[L], y[L];
+  float f;
+  crt_groups<NT, NP2, NQ4, L>(T, w, e, s, f);
+  multiple_of_P<L>(kP, min((int)rintf(f), rg_multiples(Q) - 1), y);
+  sub_limbs<L>(s, y);
+  return round_exact<L>(T, s, ex);
 }
 
 // The table of multiples q P, q < rg_multiples(Q): one uint4 each (four limbs)
@@ -888,6 +895,151 @@ __global__ void __launch_bounds__(256) reconstruct128_grouped_kernel(const __gri
   reconstruct128_entries<NP, 4>(T, i, j0, P.m, P.n, P.Y, P.ldy, P.s, P.t, P.C, P.ldc);
 }
 
+// ---------------------------------------------------------------------------
+// 16-bit digits (float formats) in groups of moduli (tables rh_* of OzTables):
+// t_g = sum_q y_q (M_g / m_q) < 2^32 per group, then the limbs, the quotient and
+// the rounding as for byte digits. Persistent, four entries per thread and task,
+// whose digits (8 bytes per channel) are copied with cp.async a task ahead. The
+// groups' sizes are template arguments (the six shapes of the frozen
+// configurations), so that the whole sum is one straight line. (In pairs of moduli:
+// twice the wide multiply-adds, and the general rounding for every entry.)
+// ---------------------------------------------------------------------------
+constexpr int kRhMultiples = 32;
+
+// The general path for one entry, from its sum's limbs.
+__device__ __noinline__ uint64_t round16_slow(const OzTables& T, const uint4* kP, const uint4 S, float f, int ex) {
+  uint32_t s[4] = {S.x, S.y, S.z, S.w}, y[4];
+  multiple_of_P<4>(kP, min((int)rintf(f), kRhMultiples - 1), y);
+  sub_limbs<4>(s, y);
+  return round_exact<4>(T, s, ex);
+}
+
+template <int... SZ>
+struct GroupSizes {
+  static constexpr int kGroups = sizeof...(SZ);
+  static constexpr int kModuli = (SZ + ...);
+  __host__ __device__ static constexpr int size(int g) {
+    const int sz[] = {SZ...};
+    return sz[g];
+  }
+  __host__ __device__ static constexpr int start(int g) {
+    const int sz[] = {SZ...};
+    int q = 0;
+    for (int i = 0; i < g; ++i) q += sz[i];
+    return q;
+  }
+};
+
+template <typename G>
+__global__ void __launch_bounds__(256, 2) reconstruct16_groups_kernel(const __grid_constant__ OzTables T, int64_t m,
+                                                                      int64_t n, const uint16_t* __restrict__ Y,
+                                                                      int64_t ldy, const int32_t* __restrict__ s,
+                                                                      const int32_t* __restrict__ t,
+                                                                      double* __restrict__ C, int64_t ldc, int64_t nch,
+                                                                      int tpr_log2) {
+  constexpr int Q = G::kModuli;
+  __shared__ uint4 kP[kRhMultiples];
+  extern __shared__ uint32_t dbuf[];                   // [2][Q][256 threads][2 words]
+  if (threadIdx.x < kRhMultiples) {
+    uint64_t carry = 0;
+    uint32_t y[4];
+#pragma unroll
+    for (int l = 0; l < 4; ++l) {
+      carry += (uint64_t)threadIdx.x * T.P[l];
+      y[l] = (uint32_t)carry;
+      carry >>= 32;
+    }
+    kP[threadIdx.x] = make_uint4(y[0], y[1], y[2], y[3]);
+  }
+  __syncthreads();
+  const int tpr = 1 << tpr_log2, rows = 256 >> tpr_log2;
+  const int r_in = threadIdx.x >> tpr_log2, c_in = threadIdx.x & (tpr - 1);
+  const int64_t plane = m * ldy;
+  const int64_t total = (m + rows - 1) / rows * nch;
+  uint32_t* const mine = dbuf + 2 * threadIdx.x;
+  auto issue = [&](int64_t b, uint32_t* buf) {
+    const int64_t i = b / nch * rows + r_in, j0 = (b % nch * tpr + c_in) * 4;
+    if (b < total && i < m && j0 < n) {
+      const uint16_t* p = Y + i * ldy + j0;
+#pragma unroll
+      for (int q = 0; q < Q; ++q) cp_async8(buf + 512 * q, reinterpret_cast<const uint32_t*>(p + q * plane));
+    }
+    cp_async_commit();
+  };
+  int slot = 0;
+  issue(blockIdx.x, mine);
+  for (int64_t b = blockIdx.x; b < total; b += gridDim.x, slot ^= 1) {
+    issue(b + gridDim.x, mine + (slot ^ 1) * Q * 512);
+    cp_async_wait1();                       // this task's copies have landed
+    const int64_t i = b / nch * rows + r_in, j0 = (b % nch * tpr + c_in) * 4;
+    if (i >= m || j0 >= n) continue;
+    const uint32_t* wsm = mine + slot * Q * 512;
+    uint2 w[Q];
+#pragma unroll
+    for (int q = 0; q < Q; ++q) w[q] = *reinterpret_cast<const uint2*>(wsm + 512 * q);
+    const int32_t si = __ldg(s + i);
+    uint64_t out[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      uint64_t a[3] = {};
+      uint32_t top = 0;
+      float f = 0.0f;
+#pragma unroll
+      for (int g = 0; g < G::kGroups; ++g) {
+        uint32_t tg = 0;
+#pragma unroll
+        for (int q = G::start(g); q < G::start(g) + G::size(g); ++q) {
+          const uint32_t x = e < 2 ? w[q].x : w[q].y;
+          tg += ((e & 1) ? x >> 16 : x & 0xffffu) * T.rh_w[q];
+        }
+#pragma unroll
+        for (int l = 0; l < 3; ++l) a[l] += (uint64_t)tg * T.rh_N[g][l];
+        top += tg * T.rh_N[g][3];
+        f = fmaf(__uint2float_rn(tg), T.rh_invM[g], f);
+      }
+      uint32_t S[4];
+      S[0] = (uint32_t)a[0];
+      asm("add.cc.u32 %0, %3, %4;\n\taddc.cc.u32 %1, %5, %6;\n\taddc.u32 %2, %7, %8;"
+          : "=r"(S[1]), "=r"(S[2]), "=r"(S[3])
+          : "r"((uint32_t)(a[0] >> 32)), "r"((uint32_t)a[1]), "r"((uint32_t)(a[1] >> 32)), "r"((uint32_t)a[2]),
+            "r"((uint32_t)(a[2] >> 32)), "r"(top));
+      const int ex = -(si + (j0 + e < n ? __ldg(t + j0 + e) : 0));
+      if (!round_groups_fast<4>(kP, kRhMultiples - 1, S, f, ex, out[e]))
+        out[e] = round16_slow(T, kP, make_uint4(S[0], S[1], S[2], S[3]), f, ex);
+    }
+    double* cp = C + i * ldc + j0;
+    if (j0 + 4 <= n && (reinterpret_cast<uintptr_t>(cp) & 15) == 0) {
+      __stcs(reinterpret_cast<double2*>(cp), make_double2(__longlong_as_double((long long)out[0]),
+                                                          __longlong_as_double((long long)out[1])));
+      __stcs(reinterpret_cast<double2*>(cp) + 1, make_double2(__longlong_as_double((long long)out[2]),
+                                                              __longlong_as_double((long long)out[3])));
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if (j0 + e < n) cp[e] = __longlong_as_double((long long)out[e]);
+    }
+  }
+}
+
+// f(GroupSizes<...>()) for the plan's groups, or cudaErrorNotSupported.
+template <typename F>
+cudaError_t with_sizes(const OzTables& T, F f) {
+  auto is = [&](auto g) {
+    using G = decltype(g);
+    if (T.rh_ng != G::kGroups || T.Q != G::kModuli) return false;
+    for (int i = 0; i < G::kGroups; ++i)
+      if (T.rh_start[i] != G::start(i)) return false;
+    return true;
+  };
+  if (is(GroupSizes<2, 2, 4, 5, 6, 1>())) return f(GroupSizes<2, 2, 4, 5, 6, 1>());
+  if (is(GroupSizes<2, 2, 2, 3, 5, 5>())) return f(GroupSizes<2, 2, 2, 3, 5, 5>());
+  if (is(GroupSizes<3, 3, 3, 5, 5>())) return f(GroupSizes<3, 3, 3, 5, 5>());
+  if (is(GroupSizes<3, 3, 3, 4, 5>())) return f(GroupSizes<3, 3, 3, 4, 5>());
+  if (is(GroupSizes<3, 3, 3, 3, 6>())) return f(GroupSizes<3, 3, 3, 3, 6>());
+  if (is(GroupSizes<3, 4, 4, 4, 6>())) return f(GroupSizes<3, 4, 4, 4, 6>());
+  return cudaErrorNotSupported;
+}
+
 template <int NP>
 cudaError_t launch128(const OzTables& T, int64_t m, int64_t n, const uint8_t* Y, int64_t ldy, const int32_t* s,
                       const int32_t* t, double* C, int64_t ldc, cudaStream_t st) {
@@ -997,6 +1149,28 @@ cudaError_t with_shape(int key, F f) {
 }
 
 }  // namespace
+
+cudaError_t launch_reconstruct16_groups(const OzTables& T, int64_t m, int64_t n, const uint16_t* Y, int64_t ldy,
+                                        const int32_t* s, const int32_t* t, double* C, int64_t ldc, cudaStream_t st) {
+  if (T.rh_ng == 0 || (ldy & 3) || (reinterpret_cast<uintptr_t>(Y) & 7)) return cudaErrorNotSupported;
+  return with_sizes(T, [&](auto sizes) {
+    using G = decltype(sizes);
+    int tpr_log2 = 5;                                  // 32 .. 256 threads per row chunk of 4 tpr entries
+    while (tpr_log2 < 8 && ((int64_t)4 << tpr_log2) < n) ++tpr_log2;
+    const int64_t rows = 256 >> tpr_log2, nch = (n + (4 << tpr_log2) - 1) / (4 << tpr_log2);
+    const int64_t total = (m + rows - 1) / rows * nch;
+    const int smem = 2 * G::kModuli * 256 * 8;
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(reconstruct16_groups_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    const int64_t grid = total < 2 * (int64_t)sms ? total : 2 * (int64_t)sms;
+    reconstruct16_groups_kernel<G><<<(unsigned)grid, 256, smem, st>>>(T, m, n, Y, ldy, s, t, C, ldc, nch, tpr_log2);
+    return cudaGetLastError();
+  });
+}
 
 // Whether the grouped reconstruct of a plan's products takes the groups'
 // kernel (eight entries per thread) rather than the pairs' (four).
