@@ -2,8 +2,11 @@
 // (Sec. "Forms and Channels"; oz_plan_fp.cpp builds the configuration).
 //
 // Reduce: for every entry and channel, the class c = a' mod m in [0, m)
-// (a' = trunc(x 2^s) from the IEEE fields, cut into 16-bit pieces, one 32-bit
-// Barrett step), then the channel's code word of c from the plan's tables:
+// (a' = trunc(x 2^s) from the IEEE fields), then the channel's code word of c.
+// Plans of at most 55 bits form the balanced residue in fp32 and look it up in a
+// table in shared memory (split_fp_rows_tab_kernel, split_fp_cols_tab_kernel);
+// wider ones cut a' into 16-bit pieces, take one 32-bit Barrett step and read the
+// plan's tables:
 // byte q of the word is the code of the plane value the form assigns to c in
 // plane q (the sign of a' selects the second half of the table, where entry r
 // holds the word of class (m - r) mod m). Planes are K-major rows: 8-bit codes
@@ -24,7 +27,8 @@
 // (W mod m) (P/m)^-1 mod m, or W mod m, as uint16.
 //
 // Reconstruct: the CRT of Sec. "Around the GEMMs" on 16-bit digits, moduli
-// taken in pairs as in oz_reconstruct.cu.
+// taken in groups whose sizes are fixed at compile time (reconstruct16_groups_kernel),
+// or in pairs as in oz_reconstruct.cu for the configurations that have none.
 #include <cuda.h>
 #include <stdint.h>
 

@@ -627,10 +627,12 @@ __global__ void __launch_bounds__(256, 3) split_cols_grouped_kernel(const __grid
 //     64-entry tiles r, r + kStripCtas, ...; it scans them for the maxima, the
 //     blocks exchange these through distributed shared memory, and each then
 //     splits its tiles (the last one from registers). No scratch, no second
-//     launch: 256^3 with the GEMM and the reconstruct in 28 us instead of 47.
+//     launch: with the dependent launches, a 256^3 product in 28-30 us instead of
+//     47 (19 since the call's host path was shortened too).
 //   Longer strided vectors: a pass for the column maxima, then 32 x 64 tiles
 //     with the shifts formed from them. (A block's tiles of a strip would run
-//     one after another, with two barriers each: 189 us against 141 us at 4096.)
+//     one after another, with two barriers each: at 4096 the shared launch takes
+//     189 us longer than the rows alone, the separate kernels for B 141 us.)
 // The passes of a small product share one launch; those of a larger one with
 // k_pad up to 1024 are launched one after another, since a shared launch costs
 // the rows L1 (65536 x 256 rows beside a 256 x 256 B: 150 us against 121 us).
