@@ -467,16 +467,18 @@ def launches_per_dgemm(trans_a: bool = False, trans_b: bool = False, engine: int
     below) split A's rows in one kernel (its columns, for trans_a, in three:
     column maxima, shifts, split) and B's columns in three (bf16 planes) or
     transposed and split as rows (two, int8 planes of the IMMA engine); one when
-    trans_b. On the TC engines a shape (m, n, k) whose padded k is at most 1024,
-    or whose padded operands have at most 2^22 entries, splits both operands
-    together: one kernel, a second one when only the first bound holds and an
-    operand's vectors are columns, and one for the tiles of longer columns."""
+    trans_b. On the TC engines a shape (m, n, k) whose padded operands have at
+    most 2^22 entries, or whose padded k is at most 1024 and whose strided
+    operands have at most 2^21, splits both operands together: one kernel, a
+    second one when only the second bound holds and an operand's vectors are
+    columns, and one for the tiles of longer columns."""
     if shape is not None and engine != OZ_ENGINE_IMMA:
         m_pad, n_pad, k_pad = round_up(shape[0], 256), round_up(shape[1], 256), round_up(shape[2], 128)
         columns = bool(trans_a) or not trans_b
         if (m_pad + n_pad) * k_pad <= 1 << 22:
             return 3 + (columns and k_pad > 1024)
-        if k_pad <= 1024:
+        strided = (m_pad if trans_a else 0) + (0 if trans_b else n_pad)
+        if k_pad <= 1024 and strided * k_pad <= 1 << 21:
             return 3 + columns
     a = 3 if trans_a else 1
     b = 1 if trans_b else (2 if engine == OZ_ENGINE_IMMA else 3)

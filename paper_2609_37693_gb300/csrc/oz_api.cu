@@ -135,7 +135,7 @@ oz_status dgemm_run(oz_plan plan, int trans_a, int trans_b, int64_t m, int64_t n
 
   // bf16 planes of small or short-vectored operands: both split together; the
   // launch clears the status word itself
-  const bool both = bf16 && oz::split_both_suits(L.m_pad, L.n_pad, L.k_pad);
+  const bool both = bf16 && oz::split_both_suits(L.m_pad, L.n_pad, L.k_pad, trans_a != 0, trans_b == 0);
   cudaError_t e = both ? cudaSuccess : cudaMemsetAsync(flag, 0, 16, st);
   if (e != cudaSuccess) return OZ_ERR_CUDA;
   if (plan->is_fp) {

@@ -1230,7 +1230,8 @@ cudaError_t launch_gemm_tc(const OzTables& t, int64_t m, int64_t n, int64_t m_pa
   if (!set_split(&p, split, ysplit)) return cudaErrorInvalidValue;
   const int64_t units = num_tiles * p.nsplit;
   const int64_t pairs = units < sms / 2 ? units : sms / 2;
-  return launch_pdl(kernel, dim3((unsigned)(2 * pairs)), dim3((2 + epi_warps) * 32), (size_t)smem_bytes, st, 1, sched, t);
+  return launch_kernel(dependent_suits(m, n), kernel, dim3((unsigned)(2 * pairs)), dim3((2 + epi_warps) * 32),
+                       (size_t)smem_bytes, st, 1, sched, t);
 }
 
 // Tensor maps of one grouped problem's planes (rows of Q planes) and its
@@ -1324,7 +1325,8 @@ cudaError_t launch_gemm_tc_single(const OzTables& t, int64_t m, int64_t n, int64
   if (!set_split(&p, split, ysplit)) return cudaErrorInvalidValue;
   const int64_t units = num_tiles * p.nsplit;
   const int grid = (int)(units < sms ? units : sms);
-  return launch_pdl(kernel, dim3((unsigned)grid), dim3(kThreads), (size_t)kSmemBytes, st, 1, mapA, mapB, t, p);
+  return launch_kernel(dependent_suits(m, n), kernel, dim3((unsigned)grid), dim3(kThreads), (size_t)kSmemBytes, st, 1,
+                       mapA, mapB, t, p);
 }
 
 }  // namespace oz

@@ -243,7 +243,8 @@ struct SplitOperand {
   void* planes;
   uint64_t* colmax;      // scratch of nvec words, for columns (each operand its own)
 };
-bool split_both_suits(int64_t m_pad, int64_t n_pad, int64_t k_pad);   // else: the splits one by one
+// else: the splits one by one
+bool split_both_suits(int64_t m_pad, int64_t n_pad, int64_t k_pad, bool a_strided, bool b_strided);
 cudaError_t launch_split_both(const OzTables& t, const SplitOperand& A, const SplitOperand& B, int64_t len,
                               int64_t k_pad, int32_t* status, cudaStream_t st);
 // The shifts of both operands as launch_split_both left them (s of m rows, t

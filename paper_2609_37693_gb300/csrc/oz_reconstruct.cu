@@ -1100,8 +1100,8 @@ cudaError_t launch_groups(const OzTables& T, int64_t m, int64_t n, const uint8_t
       return cudaErrorInvalidValue;
     int64_t grid = 2 * (int64_t)sms;                 // two blocks resident per SM (registers and digit buffers)
     if (grid > total) grid = total;
-    return launch_pdl(reconstruct_groups8_kernel<NT, NP2, NQ4>, dim3((unsigned)grid), dim3(256), (size_t)smem, st, 1, T,
-                      m, n, Y, ldy, s, t, C, ldc, nch, tpr_log2);
+    return launch_kernel(dependent_suits(m, n), reconstruct_groups8_kernel<NT, NP2, NQ4>, dim3((unsigned)grid),
+                         dim3(256), (size_t)smem, st, 1, T, m, n, Y, ldy, s, t, C, ldc, nch, tpr_log2);
   }
   int tpr_log2 = 5;                                  // 32 .. 256 threads per row chunk of 4 tpr entries
   while (tpr_log2 < 8 && ((int64_t)4 << tpr_log2) < n) ++tpr_log2;

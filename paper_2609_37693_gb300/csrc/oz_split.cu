@@ -636,8 +636,12 @@ __global__ void __launch_bounds__(256, 3) split_cols_grouped_kernel(const __grid
 // The passes of a small product share one launch; those of a larger one with
 // k_pad up to 1024 are launched one after another, since a shared launch costs
 // the rows L1 (65536 x 256 rows beside a 256 x 256 B: 150 us against 121 us).
-// Larger products of longer vectors keep the separate kernels above
-// (split_both_suits): there the launches are nothing and ld.global.nc and plain
+// Larger products of longer vectors, or of more than kStripEntries strided
+// entries, keep the separate kernels above, and launches past kMergeEntries are
+// in plain stream order (65536 x 256 x 256 with both operands transposed: 420 us
+// with separate kernels, 577 in strips, 514 before either; with neither
+// transposed 382 us in strips, 393 apart; 4096 x 4096 x 512 358 either way). In
+// long products (split_both_suits) the launches are nothing, and ld.global.nc and plain
 // launches are worth 0.8 % of an 8192^3 product.
 // ---------------------------------------------------------------------------
 struct SplitSide {
@@ -652,6 +656,7 @@ struct SplitSide {
 constexpr int kSideRow = 0, kSideWarp = 1, kSideStrip = 2, kSideTile = 3, kSideAny = -1;
 constexpr int kStripCtas = 8;
 constexpr int64_t kStripMaxK = 1024;
+constexpr int64_t kStripEntries = (int64_t)2 << 20;   // of the strided operands of a larger product
 constexpr int64_t kMergeEntries = (int64_t)4 << 20;   // of both operands: up to which their passes share a launch
 
 template <int NP, int QT>
@@ -876,16 +881,18 @@ cudaError_t split_both_qt(const OzTables& t, const SplitSide& a, const SplitSide
       if (e != cudaSuccess) return e;
     }
   cudaError_t e = cudaSuccess;
+  const bool small = (a.nvec_pad + b.nvec_pad) * k_pad <= kMergeEntries;
   // one launch of the sides x, y (either may be empty)
   auto first = [&](SplitSide x, SplitSide y) {
     if (e != cudaSuccess || x.blocks1 + y.blocks1 == 0) return;
     const bool strips = (x.blocks1 && x.kind == kSideStrip) || (y.blocks1 && y.kind == kSideStrip);
     const bool warps = (!x.blocks1 || x.kind == kSideWarp) && (!y.blocks1 || y.kind == kSideWarp);
-    e = launch_pdl(warps ? split_both_kernel<NP, QT, kSideWarp> : split_both_kernel<NP, QT, kSideAny>, dim3((unsigned)(x.blocks1 + y.blocks1)), dim3(256), strips ? (size_t)tile : 0, st,
-                   strips ? kStripCtas : 1, t, x, y, len, k_pad, status);
+    e = launch_kernel(small, warps ? split_both_kernel<NP, QT, kSideWarp> : split_both_kernel<NP, QT, kSideAny>,
+                      dim3((unsigned)(x.blocks1 + y.blocks1)), dim3(256), strips ? (size_t)tile : 0, st,
+                      strips ? kStripCtas : 1, t, x, y, len, k_pad, status);
     status = nullptr;
   };
-  if ((a.nvec_pad + b.nvec_pad) * k_pad <= kMergeEntries || (a.kind == kSideWarp && b.kind == kSideWarp)) {
+  if (small || (a.kind == kSideWarp && b.kind == kSideWarp)) {
     first(a, b);
   } else {
     const SplitSide none = {};
@@ -893,8 +900,8 @@ cudaError_t split_both_qt(const OzTables& t, const SplitSide& a, const SplitSide
     first(a, none);
   }
   if (e != cudaSuccess || a.blocks2 + b.blocks2 == 0) return e;
-  return launch_pdl(split_tiles_kernel<NP, QT>, dim3((unsigned)(a.blocks2 + b.blocks2)), dim3(256), (size_t)tile, st, 1,
-                    t, a, b, len, k_pad);
+  return launch_kernel(small, split_tiles_kernel<NP, QT>, dim3((unsigned)(a.blocks2 + b.blocks2)), dim3(256),
+                       (size_t)tile, st, 1, t, a, b, len, k_pad);
 }
 
 SplitSide split_side(const SplitOperand& o, int64_t len, int64_t k_pad) {
@@ -921,8 +928,9 @@ SplitSide split_side(const SplitOperand& o, int64_t len, int64_t k_pad) {
 
 }  // namespace
 
-bool split_both_suits(int64_t m_pad, int64_t n_pad, int64_t k_pad) {
-  return k_pad <= kStripMaxK || (m_pad + n_pad) * k_pad <= kMergeEntries;
+bool split_both_suits(int64_t m_pad, int64_t n_pad, int64_t k_pad, bool a_strided, bool b_strided) {
+  const int64_t strided = (a_strided ? m_pad : 0) + (b_strided ? n_pad : 0);
+  return (m_pad + n_pad) * k_pad <= kMergeEntries || (k_pad <= kStripMaxK && strided * k_pad <= kStripEntries);
 }
 
 cudaError_t launch_split_both(const OzTables& t, const SplitOperand& A, const SplitOperand& B, int64_t len,

@@ -48,6 +48,19 @@ def test_split_routes_match_oracle(m, n, k, ta, tb):
     assert_oracle_bits(C, A, B, plan.moduli, plan.bits, what=f"{m}x{n}x{k} ta={ta} tb={tb}", count=600)
 
 
+# either side of the most strided entries that are split together, and of the
+# largest output whose kernels are launched dependent
+@pytest.mark.parametrize("m,n,k,ta,tb", [(16300, 40, 256, 0, 0), (16300, 40, 256, 1, 0), (40, 16300, 256, 0, 0),
+                                         (40, 16300, 256, 0, 1), (8200, 8200, 250, 1, 1), (4095, 2048, 64, 0, 0),
+                                         (4096, 2048, 64, 0, 0)])
+def test_routes_of_large_products_of_short_vectors(m, n, k, ta, tb):
+    plan = oz.Plan(16, 0, k)
+    A, B, Ad, Bd = _operands(m, n, k, ta, tb, m + k)
+    C = oz.dgemm(Ad, Bd, plan, trans_a=bool(ta), trans_b=bool(tb))
+    torch.cuda.synchronize()
+    assert_oracle_bits(C, A, B, plan.moduli, plan.bits, what=f"{m}x{n}x{k} ta={ta} tb={tb}", count=600)
+
+
 @pytest.mark.parametrize("q,bits", [(14, 0), (18, 62), (20, 70), (19, 66)])
 @pytest.mark.parametrize("k", [200, 1500])
 def test_split_routes_of_every_piece_count(q, bits, k):
