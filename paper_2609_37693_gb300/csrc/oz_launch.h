@@ -12,10 +12,11 @@ namespace oz {
 
 // Outputs from this many entries on are launched in plain stream order. A
 // dependent launch is worth 2 us at 2048^3 (285 against 287) and most of the
-// gaps of a small product, but cost a large one more than that: 65536 x 256 x 256
+// gaps of a small product, but cost a larger one more than that: 2400 x 2400 x
+// 512 200 us against 191, 3000 x 2500 x 2000 507 against 499, 65536 x 256 x 256
 // 390 us against 382, 8192 x 8192 x 256 1001 against 978, 16384^3 94.9 ms
 // against 94.3.
-constexpr int64_t kDependentMaxOutput = 8ll << 20;
+constexpr int64_t kDependentMaxOutput = 5ll << 20;
 
 // Whether the GEMM and the reconstruct of an m x n output are launched dependent.
 inline bool dependent_suits(int64_t m, int64_t n) { return n == 0 || m < kDependentMaxOutput / n; }

@@ -52,7 +52,7 @@ def test_split_routes_match_oracle(m, n, k, ta, tb):
 # largest output whose kernels are launched dependent
 @pytest.mark.parametrize("m,n,k,ta,tb", [(16300, 40, 256, 0, 0), (16300, 40, 256, 1, 0), (40, 16300, 256, 0, 0),
                                          (40, 16300, 256, 0, 1), (8200, 8200, 250, 1, 1), (4095, 2048, 64, 0, 0),
-                                         (4096, 2048, 64, 0, 0)])
+                                         (4096, 2048, 64, 0, 0), (2559, 2048, 64, 0, 0), (2560, 2048, 64, 0, 0)])
 def test_routes_of_large_products_of_short_vectors(m, n, k, ta, tb):
     plan = oz.Plan(16, 0, k)
     A, B, Ad, Bd = _operands(m, n, k, ta, tb, m + k)
