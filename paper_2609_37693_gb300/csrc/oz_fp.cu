@@ -306,14 +306,16 @@ __device__ __forceinline__ Pieces11 pieces11(uint64_t bits, int32_t s) {
   return P;
 }
 
-// The code words of eight entries in channel c; tab: the table's shared address.
-__device__ __forceinline__ void table_words(const OzFpTables& F, int c, uint32_t tab, const Pieces11 (&P)[8],
+// The code words of eight entries in channel c; tab: the table in shared memory
+// (read through the pointer, so that the look-ups stay behind the barrier that
+// publishes it).
+__device__ __forceinline__ void table_words(const OzFpTables& F, int c, const uint32_t* tab, const Pieces11 (&P)[8],
                                             uint32_t (&w)[8]) {
   const float2 kC = make_float2(12582912.0f, 12582912.0f), kCn = make_float2(-12582912.0f, -12582912.0f);
   const float2 inv = make_float2(F.invm[c], F.invm[c]), nm = make_float2(-F.mf[c], -F.mf[c]);
   const float2 c0 = make_float2(F.c11f[0][c], F.c11f[0][c]), c1 = make_float2(F.c11f[1][c], F.c11f[1][c]),
                c2 = make_float2(F.c11f[2][c], F.c11f[2][c]);
-  const uint32_t base = tab + 4u * (F.ch_coff[c] - 0x4B400000u);     // word of residue 0, less 4 * bits(1.5 * 2^23)
+  const uint32_t base = F.ch_coff[c] - 0x4B400000u;                  // index of residue 0, less bits(1.5 * 2^23)
 #pragma unroll
   for (int e = 0; e < 8; e += 2) {
     float2 y = make_float2(P[e].p[0], P[e + 1].p[0]);
@@ -322,15 +324,14 @@ __device__ __forceinline__ void table_words(const OzFpTables& F, int c, uint32_t
     y = __ffma2_rn(make_float2(P[e].p[3], P[e + 1].p[3]), c2, y);
     const float2 q = __fadd2_rn(__ffma2_rn(y, inv, kC), kCn);
     const float2 r = __fadd2_rn(__ffma2_rn(q, nm, y), kC);
-    asm("ld.shared.u32 %0, [%1];" : "=r"(w[e]) : "r"(base + 4u * __float_as_uint(r.x)));
-    asm("ld.shared.u32 %0, [%1];" : "=r"(w[e + 1]) : "r"(base + 4u * __float_as_uint(r.y)));
+    w[e] = tab[base + __float_as_uint(r.x)];
+    w[e + 1] = tab[base + __float_as_uint(r.y)];
   }
 }
 
-__device__ __forceinline__ uint32_t load_code_table(const OzFpTables& F, uint32_t* sm) {
+__device__ __forceinline__ void load_code_table(const OzFpTables& F, uint32_t* sm) {
   for (int i = threadIdx.x; i < F.cw_total; i += (int)blockDim.x) sm[i] = __ldg(F.cwords + i);
   __syncthreads();
-  return smem_u32(sm);
 }
 
 template <int CB>
@@ -344,7 +345,7 @@ __global__ void __launch_bounds__(256, 3) split_fp_rows_tab_kernel(const __grid_
   extern __shared__ uint32_t code_tab[];
   __shared__ uint64_t red[8];
   __shared__ int32_t s_sh;
-  const uint32_t tab = load_code_table(F, code_tab);
+  load_code_table(F, code_tab);
   const int tid = threadIdx.x;
   const int64_t row_bytes = CB == 4 ? k_pad / 2 : k_pad;
   const int64_t plane = nvec_pad * row_bytes;
@@ -400,7 +401,7 @@ __global__ void __launch_bounds__(256, 3) split_fp_rows_tab_kernel(const __grid_
       for (int e = 0; e < 8; ++e) P[e] = pieces11(b[e], s);
       for (int c = 0; c < F.nch; ++c) {
         uint32_t w[8];
-        table_words(F, c, tab, P, w);
+        table_words(F, c, code_tab, P, w);
         const int p0 = F.ch_plane0[c], np = F.ch_nplanes[c];
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
@@ -445,7 +446,7 @@ __global__ void __launch_bounds__(kFpColThreads, 2) split_fp_cols_tab_kernel(con
   uint8_t* const stage = reinterpret_cast<uint8_t*>(fp_smem);
   uint32_t* const code_tab = reinterpret_cast<uint32_t*>(stage + 6 * kFpStagePlane);
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  const uint32_t tab = load_code_table(F, code_tab);
+  load_code_table(F, code_tab);
   const int64_t row_bytes = CB == 4 ? k_pad / 2 : k_pad;
   const int64_t plane = nvec_pad * row_bytes;
   const uint64_t* Xb = reinterpret_cast<const uint64_t*>(X);
@@ -465,7 +466,7 @@ __global__ void __launch_bounds__(kFpColThreads, 2) split_fp_cols_tab_kernel(con
     uint8_t* const out = planes + j0 * row_bytes + (CB == 4 ? hbase / 2 : hbase);
     for (int c = 0; c < F.nch; ++c, turn ^= 1u) {
       uint32_t wd[8];
-      table_words(F, c, tab, P, wd);
+      table_words(F, c, code_tab, P, wd);
       const int p0 = F.ch_plane0[c], np = F.ch_nplanes[c];
       uint8_t* const buf = stage + turn * 3 * kFpStagePlane;
 #pragma unroll
