@@ -458,7 +458,7 @@ __global__ void __launch_bounds__(256) reconstruct128_kernel(const __grid_consta
 }
 
 // ---------------------------------------------------------------------------
-// Byte digits in groups of moduli (Q <= 16; tables rg_* of OzTables).
+// Byte digits in groups of moduli (Q <= 20; tables rg_* of OzTables).
 // ---------------------------------------------------------------------------
 
 // t_g of group g for entry e of the digit words w (byte e of each word is that
@@ -547,78 +547,151 @@ __device__ __forceinline__ void multiple_of_P(const uint4* kP, int q, uint32_t (
   if constexpr (L == 5) y[4] = kP[2 * q + 1].x;
 }
 
-// fl(X 2^ex) for X = S - qP, q the quotient estimate, in the usual case: the
-// estimate clear of a tie, |X| >= 2^64 and a normal result. It runs in 32-bit
-// limbs: the magnitude by a sign mask, moved up whole limbs until the top one is
-// not zero (once for four limbs: products of operands of a wide exponent spread
-// often stay below 2^96, and every one left to the general path cost its warp;
-// 4096^2 at phi = 4 108 us instead of 232, and 108 instead of 103 at phi = 0.5),
-// the leading bit by clz, 64 bits below it by funnel shifts, one
-// round-to-nearest-even increment (a carry out of the significand bumps the
-// exponent field, up to infinity). Returns false (out unset) otherwise.
+// out[e] = fl(X 2^ex) of four entries, X = S - qP with q the quotient estimate,
+// unless the estimate is next to a tie: returns a bit for each entry of these
+// (its out unset). It runs in 32-bit limbs: the magnitude by a sign mask, its four
+// limbs from the leading one down, the leading bit by clz, 64 bits below it by
+// funnel shifts, one round-to-nearest-even increment (a carry out of the
+// significand bumps the exponent field, up to infinity).
+//   What an ordinary entry does not need stands in branches taken once for the
+// four: limbs are moved up when a top limb is zero (operands of a wide
+// exponent spread give products far below the widest, few moduli give short
+// ones), one limb first and two more only below 2^64; zeros, overflow and
+// subnormal results are formed from the same limbs. A move that every entry pays
+// for costs more, and so does leaving these to the general path (oz_reconstruct
+// at 4096^2, us: no moves here, one move for every entry, and as it is now):
+//   Q = 16, phi 0.5    103  110   99      Q = 9, phi 0.5        248  331   93
+//   Q = 16, phi 4      155  110  101      Q = 16, all subnormal 298  382  125
+//   Q = 12, phi 0.5    268   96   95      E4M3, all subnormal   199  394  162
+// (E4M3's 199: moduli in pairs, every entry on the general path.)
 template <int L>
-__device__ __forceinline__ bool round_groups_fast(const uint4* kP, int kmax, const uint32_t (&s)[L], float f, int ex,
-                                                  uint64_t& out) {
-  const float kf = rintf(f);
-  uint32_t m[L], y[L];
-  // digits past n in a row's padding are whatever the workspace holds, and their
-  // quotient may lie past the table: kmax, its last multiple
-  multiple_of_P<L>(kP, min((int)kf, kmax), y);
+__device__ __forceinline__ uint32_t round4_fast(const uint4* kP, int kmax, const uint32_t (&S)[4][L],
+                                                const float (&f)[4], int (&ex)[4], uint64_t (&out)[4]) {
+  uint32_t h[4][4], low[4], neg[4];           // h[e][3]: the top limb; low: bits below the four
+  uint32_t slow = 0, zero = 0, least = 0xffffffffu;
 #pragma unroll
-  for (int l = 0; l < L; ++l) m[l] = s[l];
-  sub_limbs<L>(m, y);
-  // magnitude: (x ^ mask) - mask
-  const uint32_t mask = (uint32_t)((int32_t)m[L - 1] >> 31);
+  for (int e = 0; e < 4; ++e) {
+    const float kf = rintf(f[e]);
+    uint32_t m[L], y[L];
+    // digits past n in a row's padding are whatever the workspace holds, and their
+    // quotient may lie past the table: kmax, its last multiple
+    multiple_of_P<L>(kP, min((int)kf, kmax), y);
 #pragma unroll
-  for (int l = 0; l < L; ++l) m[l] ^= mask, y[l] = mask;
-  sub_limbs<L>(m, y);
-  uint32_t low = 0;                                        // bits below the four limbs rounded
-  int top = 127;
-  if constexpr (L == 5) {
-    if (m[4] != 0) {
-      low = m[0], m[0] = m[1], m[1] = m[2], m[2] = m[3], m[3] = m[4];
-      top = 159;
+    for (int l = 0; l < L; ++l) m[l] = S[e][l];
+    sub_limbs<L>(m, y);
+    slow |= (uint32_t)(fabsf(f[e] - kf) > 0.499f) << e;
+    // magnitude: (x ^ mask) - mask
+    const uint32_t mask = (uint32_t)((int32_t)m[L - 1] >> 31);
+    neg[e] = mask & 0x80000000u;
+#pragma unroll
+    for (int l = 0; l < L; ++l) m[l] ^= mask, y[l] = mask;
+    sub_limbs<L>(m, y);
+    low[e] = 0;
+    if constexpr (L == 5) {
+      if (m[4] != 0) {
+        low[e] = m[0], m[0] = m[1], m[1] = m[2], m[2] = m[3], m[3] = m[4];
+        ex[e] += 32;
+      }
+    }
+#pragma unroll
+    for (int l = 0; l < 4; ++l) h[e][l] = m[l];
+    least = min(least, m[3]);
+  }
+  if (least == 0) {
+    auto move_up = [&](int e) {
+      if (h[e][3] == 0) {
+        h[e][3] = h[e][2], h[e][2] = h[e][1], h[e][1] = h[e][0], h[e][0] = 0u;
+        ex[e] -= 32;
+      }
+    };
+    least = 0xffffffffu;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      move_up(e);
+      least = min(least, h[e][3]);
+    }
+    if (least == 0) {                                        // some |X| < 2^64
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        move_up(e);
+        move_up(e);
+        zero |= (uint32_t)(h[e][3] == 0) << e;
+      }
     }
   }
-  if (m[3] == 0) {
-    m[3] = m[2], m[2] = m[1], m[1] = m[0], m[0] = 0u;
-    top = 95;
+  uint32_t range = 0;
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    const int lz = __clz((int)h[e][3]);
+    const int E = 127 - lz + ex[e];                          // exponent of the leading bit
+    range |= (uint32_t)((unsigned)(E + 1022) > 2045u) << e;
+    // 64 bits from the leading one down (h1:h0), and whether any bit below is set
+    const uint32_t h1 = __funnelshift_l(h[e][2], h[e][3], lz);
+    const uint32_t h0 = __funnelshift_l(h[e][1], h[e][2], lz);
+    const uint32_t r = __funnelshift_l(h[e][0], h[e][1], lz) | (h[e][0] << lz) | low[e];
+    const uint64_t mant = (((uint64_t)h1 << 32) | h0) >> 11;  // 53 bits, leading one at bit 52
+    const uint32_t half = (h0 >> 10) & 1u;
+    const uint32_t sticky = ((h0 & 0x3ffu) | r) != 0u;
+    const uint64_t q = mant + (half & (sticky | (uint32_t)mant));
+    out[e] = (((uint64_t)(E + 1022) << 52) + q) | ((uint64_t)neg[e] << 32);
   }
-  const int lz = __clz((int)m[3]);
-  const int E = top - lz + ex;                             // exponent of the leading bit
-  if (fabsf(f - kf) > 0.499f || m[3] == 0 || (unsigned)(E + 1022) > 2045u) return false;
-  // 64 bits from the leading one down (h1:h0), and whether any bit below is set
-  const uint32_t h1 = __funnelshift_l(m[2], m[3], lz);
-  const uint32_t h0 = __funnelshift_l(m[1], m[2], lz);
-  const uint32_t r = __funnelshift_l(m[0], m[1], lz) | (m[0] << lz) | low;
-  const uint64_t mant = (((uint64_t)h1 << 32) | h0) >> 11;  // 53 bits, leading one at bit 52
-  const uint32_t half = (h0 >> 10) & 1u;
-  const uint32_t sticky = ((h0 & 0x3ffu) | r) != 0u;
-  const uint64_t q = mant + (half & (sticky | (uint32_t)mant));
-  out = (((uint64_t)(E + 1022) << 52) + q) | ((uint64_t)(mask & 0x80000000u) << 32);
-  return true;
+  if (range) {                                               // overflow, subnormal results and those below
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      if (!((range >> e) & 1u)) continue;
+      const int lz = __clz((int)h[e][3]);
+      const int E = 127 - lz + ex[e];
+      uint64_t q = 0x7ff0000000000000ull;
+      if (E < 0) {
+        const uint64_t M = ((uint64_t)__funnelshift_l(h[e][2], h[e][3], lz) << 32) | __funnelshift_l(h[e][1], h[e][2], lz);
+        const uint32_t r = __funnelshift_l(h[e][0], h[e][1], lz) | (h[e][0] << lz) | low[e];
+        const int sh = -1011 - E;                            // bits of M below 2^-1074: 12 or more
+        q = sh < 64 ? M >> sh : 0ull;
+        const uint64_t rest = sh < 64 ? M << (64 - sh) : sh == 64 ? M : 0ull;   // the half bit on top
+        if ((rest >> 63) && ((rest << 1) | r | (q & 1ull))) ++q;
+      }
+      out[e] = q | ((uint64_t)neg[e] << 32);
+    }
+  }
+  if (zero) {                                                // X = 0 gives +0
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      if ((zero >> e) & 1u) out[e] = 0ull;
+    slow &= ~zero;
+  }
+  return slow;
 }
 
 // fl(X 2^ex) of the candidate X in s (two's complement, |X| < 3P/2), corrected
-// exactly into [-P/2, P/2), by the general rounding.
+// exactly into [-P/2, P/2), by the general rounding (four limbs: in 128-bit
+// integers).
 template <int L>
 __device__ __forceinline__ uint64_t round_exact(const OzTables& T, const uint32_t (&s)[L], int ex) {
-  Limbs<L> X;
+  if constexpr (L == 4) {
+    __int128 X = (__int128)(((u128)(((uint64_t)s[3] << 32) | s[2]) << 64) | (((uint64_t)s[1] << 32) | s[0]));
+    const u128 P = ((u128)(((uint64_t)T.P[3] << 32) | T.P[2]) << 64) | (((uint64_t)T.P[1] << 32) | T.P[0]);
+    if (2 * X >= (__int128)P) X -= (__int128)P;
+    else if (2 * X < -(__int128)P) X += (__int128)P;
+    const uint32_t neg = X < 0;
+    return round128(neg ? (u128)(-X) : (u128)X, neg, ex);
+  } else {
+    Limbs<L> X;
 #pragma unroll
-  for (int l = 0; l < L; ++l) X.w[l] = s[l];
-  if (twice_ge_P(X, T.P)) sub_mul_P(X, 1u, T.P);
-  else if (twice_lt_minus_P(X, T.P)) add_P(X, T.P);
-  const uint32_t neg = X.w[L - 1] >> 31;
-  if (neg) {
-    uint64_t c = 1;
+    for (int l = 0; l < L; ++l) X.w[l] = s[l];
+    if (twice_ge_P(X, T.P)) sub_mul_P(X, 1u, T.P);
+    else if (twice_lt_minus_P(X, T.P)) add_P(X, T.P);
+    const uint32_t neg = X.w[L - 1] >> 31;
+    if (neg) {
+      uint64_t c = 1;
 #pragma unroll
-    for (int l = 0; l < L; ++l) {
-      const uint64_t v = (uint64_t)(~X.w[l]) + c;
-      X.w[l] = (uint32_t)v;
-      c = v >> 32;
+      for (int l = 0; l < L; ++l) {
+        const uint64_t v = (uint64_t)(~X.w[l]) + c;
+        X.w[l] = (uint32_t)v;
+        c = v >> 32;
+      }
     }
+    return round_to_binary64(X, neg, ex);
   }
-  return round_to_binary64(X, neg, ex);
 }
 
 // Every other case, recomputed from the digits (wsm[q * QS], this thread's
@@ -682,14 +755,15 @@ __device__ __forceinline__ void rec4_groups(const OzTables& T, const uint4* kP, 
 #pragma unroll
   for (int q = 0; q < Q; ++q) w[q] = wsm[q * QS];
   uint64_t out[4];
-  uint32_t slow = 0;
+  uint32_t S[4][L];
+  float f[4];
+  int ex[4];
 #pragma unroll
   for (int e = 0; e < 4; ++e) {
-    uint32_t S[L];
-    float f;
-    crt_groups<NT, NP2, NQ4, L>(T, w, e, S, f);
-    if (!round_groups_fast<L>(kP, rg_multiples(Q) - 1, S, f, -(si + tj[e]), out[e])) slow |= 1u << e;
+    crt_groups<NT, NP2, NQ4, L>(T, w, e, S[e], f[e]);
+    ex[e] = -(si + tj[e]);
   }
+  const uint32_t slow = round4_fast<L>(kP, rg_multiples(Q) - 1, S, f, ex, out);
   if (slow) {                                              // rare: one branch for the four entries
 #pragma unroll
     for (int e = 0; e < 4; ++e)
@@ -853,11 +927,12 @@ __global__ void __launch_bounds__(256, 2) reconstruct_groups8_kernel(const __gri
 // that short rows share a block; eight entries per thread, as in
 // reconstruct_groups8_kernel), with the groups' sum. (A persistent form with a
 // task of lookahead, as reconstruct_groups_kernel, ran the 256-product batch
-// 3-8 % slower at four entries per thread.)
+// 3-8 % slower at four entries per thread.) Four blocks per SM up to 16 moduli:
+// 256-product batch 13.68 ms, 13.83 with the 66 registers that leave three.
 template <int NT, int NP2, int NQ4>
-__global__ void __launch_bounds__(256) reconstruct_groups_grouped_kernel(const __grid_constant__ OzTables T,
-                                                                         const OzGroupProblem* __restrict__ probs,
-                                                                         const int32_t* __restrict__ map) {
+__global__ void __launch_bounds__(256, 3 * NT + 2 * NP2 + 4 * NQ4 <= 16 ? 4 : 3)
+reconstruct_groups_grouped_kernel(const __grid_constant__ OzTables T, const OzGroupProblem* __restrict__ probs,
+                                  const int32_t* __restrict__ map) {
   constexpr int Q = 3 * NT + 2 * NP2 + 4 * NQ4;
   __shared__ MultiplesOfP<Q> kPs;
   extern __shared__ uint32_t dbuf[];                   // [Q][256 threads][2 words]
@@ -907,14 +982,6 @@ __global__ void __launch_bounds__(256) reconstruct128_grouped_kernel(const __gri
 // ---------------------------------------------------------------------------
 constexpr int kRhMultiples = 32;
 
-// The general path for one entry, from its sum's limbs.
-__device__ __noinline__ uint64_t round16_slow(const OzTables& T, const uint4* kP, const uint4 S, float f, int ex) {
-  uint32_t s[4] = {S.x, S.y, S.z, S.w}, y[4];
-  multiple_of_P<4>(kP, min((int)rintf(f), kRhMultiples - 1), y);
-  sub_limbs<4>(s, y);
-  return round_exact<4>(T, s, ex);
-}
-
 template <int... SZ>
 struct GroupSizes {
   static constexpr int kGroups = sizeof...(SZ);
@@ -930,6 +997,45 @@ struct GroupSizes {
     return q;
   }
 };
+
+// The CRT sum of entry e of the digit words w(q) (two words of two digits each):
+// S modulo 2^128 and the estimate f of S / P, as crt_groups.
+template <typename G, typename W>
+__device__ __forceinline__ void crt16_groups(const OzTables& T, W w, int e, uint32_t (&S)[4], float& f) {
+  uint64_t a[3] = {};
+  uint32_t top = 0;
+  f = 0.0f;
+#pragma unroll
+  for (int g = 0; g < G::kGroups; ++g) {
+    uint32_t tg = 0;
+#pragma unroll
+    for (int q = G::start(g); q < G::start(g) + G::size(g); ++q) {
+      const uint2 v = w(q);
+      const uint32_t x = e < 2 ? v.x : v.y;
+      tg += ((e & 1) ? x >> 16 : x & 0xffffu) * T.rh_w[q];
+    }
+#pragma unroll
+    for (int l = 0; l < 3; ++l) a[l] += (uint64_t)tg * T.rh_N[g][l];
+    top += tg * T.rh_N[g][3];
+    f = fmaf(__uint2float_rn(tg), T.rh_invM[g], f);
+  }
+  S[0] = (uint32_t)a[0];
+  asm("add.cc.u32 %0, %3, %4;\n\taddc.cc.u32 %1, %5, %6;\n\taddc.u32 %2, %7, %8;"
+      : "=r"(S[1]), "=r"(S[2]), "=r"(S[3])
+      : "r"((uint32_t)(a[0] >> 32)), "r"((uint32_t)a[1]), "r"((uint32_t)(a[1] >> 32)), "r"((uint32_t)a[2]),
+        "r"((uint32_t)(a[2] >> 32)), "r"(top));
+}
+
+// The general path for one entry, from the digits in this thread's slots.
+template <typename G>
+__device__ __noinline__ uint64_t round16_slow(const OzTables& T, const uint4* kP, const uint32_t* wsm, int e, int ex) {
+  uint32_t s[4], y[4];
+  float f;
+  crt16_groups<G>(T, [&](int q) { return *reinterpret_cast<const uint2*>(wsm + 512 * q); }, e, s, f);
+  multiple_of_P<4>(kP, min((int)rintf(f), kRhMultiples - 1), y);
+  sub_limbs<4>(s, y);
+  return round_exact<4>(T, s, ex);
+}
 
 template <typename G>
 __global__ void __launch_bounds__(256, 2) reconstruct16_groups_kernel(const __grid_constant__ OzTables T, int64_t m,
@@ -980,33 +1086,20 @@ __global__ void __launch_bounds__(256, 2) reconstruct16_groups_kernel(const __gr
     for (int q = 0; q < Q; ++q) w[q] = *reinterpret_cast<const uint2*>(wsm + 512 * q);
     const int32_t si = __ldg(s + i);
     uint64_t out[4];
+    uint32_t S[4][4];
+    float f[4];
+    int ex[4], tj[4];
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-      uint64_t a[3] = {};
-      uint32_t top = 0;
-      float f = 0.0f;
+      crt16_groups<G>(T, [&](int q) { return w[q]; }, e, S[e], f[e]);
+      tj[e] = j0 + e < n ? __ldg(t + j0 + e) : 0;
+      ex[e] = -(si + tj[e]);
+    }
+    const uint32_t slow = round4_fast<4>(kP, kRhMultiples - 1, S, f, ex, out);
+    if (slow) {
 #pragma unroll
-      for (int g = 0; g < G::kGroups; ++g) {
-        uint32_t tg = 0;
-#pragma unroll
-        for (int q = G::start(g); q < G::start(g) + G::size(g); ++q) {
-          const uint32_t x = e < 2 ? w[q].x : w[q].y;
-          tg += ((e & 1) ? x >> 16 : x & 0xffffu) * T.rh_w[q];
-        }
-#pragma unroll
-        for (int l = 0; l < 3; ++l) a[l] += (uint64_t)tg * T.rh_N[g][l];
-        top += tg * T.rh_N[g][3];
-        f = fmaf(__uint2float_rn(tg), T.rh_invM[g], f);
-      }
-      uint32_t S[4];
-      S[0] = (uint32_t)a[0];
-      asm("add.cc.u32 %0, %3, %4;\n\taddc.cc.u32 %1, %5, %6;\n\taddc.u32 %2, %7, %8;"
-          : "=r"(S[1]), "=r"(S[2]), "=r"(S[3])
-          : "r"((uint32_t)(a[0] >> 32)), "r"((uint32_t)a[1]), "r"((uint32_t)(a[1] >> 32)), "r"((uint32_t)a[2]),
-            "r"((uint32_t)(a[2] >> 32)), "r"(top));
-      const int ex = -(si + (j0 + e < n ? __ldg(t + j0 + e) : 0));
-      if (!round_groups_fast<4>(kP, kRhMultiples - 1, S, f, ex, out[e]))
-        out[e] = round16_slow(T, kP, make_uint4(S[0], S[1], S[2], S[3]), f, ex);
+      for (int e = 0; e < 4; ++e)
+        if ((slow >> e) & 1u) out[e] = round16_slow<G>(T, kP, wsm, e, -(si + tj[e]));
     }
     double* cp = C + i * ldc + j0;
     if (j0 + 4 <= n && (reinterpret_cast<uintptr_t>(cp) & 15) == 0) {
