@@ -412,8 +412,9 @@ def dgemm(A, B, plan: Plan | None = None, trans_a: bool = False, trans_b: bool =
         C, ldc = out, _ld(out)
     if ws is None:
         ws = workspace(plan, m, n, k, A.device)
-    st = _lib.oz_dgemm(plan.handle, 1 if trans_a else 0, 1 if trans_b else 0, m, n, k, A.data_ptr(), lda,
-                       B.data_ptr(), ldb, C.data_ptr(), ldc, ws.data_ptr(), ws.numel(),
+    # the flags as they are: the library refuses all but 0 and 1
+    st = _lib.oz_dgemm(plan.handle, int(trans_a), int(trans_b), m, n, k, A.data_ptr(), lda, B.data_ptr(), ldb,
+                       C.data_ptr(), ldc, ws.data_ptr(), ws.numel(),
                        _raw_stream() if stream is None else stream.cuda_stream)
     if st != OZ_OK:
         raise OzError(st, "oz_dgemm")
