@@ -493,6 +493,15 @@ OZ_API oz_status oz_static_query_status(void* stream);
  */
 OZ_API oz_status oz_selftest_bounded_wait(int arrive, int32_t* status, void* stream);
 
+/*
+ * oz_selftest_digit16_groups -- the groups of moduli that a float-format plan's
+ * reconstruct takes together: *groups of them (0: moduli in pairs instead),
+ * group g the moduli starts[g] .. starts[g + 1] - 1 (starts: at least 9 ints);
+ * *compiled 1 if the kernel exists for these sizes (else moduli in pairs).
+ * Host only.
+ */
+OZ_API oz_status oz_selftest_digit16_groups(oz_plan plan, int* groups, int* starts, int* compiled);
+
 /* Short English description of a status code (static string). */
 OZ_API const char* oz_status_str(oz_status status);
 

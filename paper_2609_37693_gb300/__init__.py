@@ -54,7 +54,7 @@ EXPORTED = ("oz_plan_create", "oz_plan_info", "oz_plan_destroy", "oz_workspace_b
             "oz_dgemm_host", "oz_plan_create_fp", "oz_plan_info_fp", "oz_plane_geometry",
             "oz_grouped_workspace_bytes", "oz_group_create", "oz_group_run", "oz_group_destroy",
             "oz_plan_caps", "oz_blocked_workspace_bytes", "oz_dgemm_blocked", "oz_selftest_bounded_wait",
-            "oz_transpose", "oz_static_query_status")
+            "oz_transpose", "oz_static_query_status", "oz_selftest_digit16_groups")
 
 
 class OzError(RuntimeError):
@@ -104,6 +104,7 @@ def _load_library():
         "oz_dgemm_blocked": (I32, [P, I32, I32, I64, I64, I64, I64, P, I64, P, I64, P, I64, P, SZ, P]),
         "oz_selftest_bounded_wait": (I32, [I32, P, P]),
         "oz_transpose": (I32, [I64, I64, P, I64, P, P]),
+        "oz_selftest_digit16_groups": (I32, [P, P, P, P]),
     }
     for name, (res, args) in sig.items():
         f = getattr(lib, name)
@@ -263,6 +264,14 @@ def oz_selftest_bounded_wait(arrive, status, stream) -> int:
     """status: device pointer to an int32 (OR-ed with 4 if the wait completed,
     2 if it ran out)."""
     return _lib.oz_selftest_bounded_wait(int(arrive), status, stream)
+
+
+def oz_selftest_digit16_groups(plan):
+    """(status, first modulus of each group and the modulus count, whether the
+    grouped kernel is compiled for these sizes) of a float-format plan."""
+    groups, starts, compiled = ctypes.c_int(), (ctypes.c_int * 9)(), ctypes.c_int()
+    st = _lib.oz_selftest_digit16_groups(plan, ctypes.byref(groups), starts, ctypes.byref(compiled))
+    return st, list(starts[:groups.value + 1]), bool(compiled.value)
 
 
 def oz_transpose(rows, cols, X, ld, Y, stream) -> int:

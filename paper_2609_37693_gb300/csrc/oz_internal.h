@@ -313,6 +313,8 @@ cudaError_t launch_reconstruct16(const OzTables& t, int64_t m, int64_t n, const 
 // plan's tables or Y's pitch and base (multiples of 4 digits) do not serve it
 cudaError_t launch_reconstruct16_groups(const OzTables& t, int64_t m, int64_t n, const uint16_t* Y, int64_t ldy,
                                         const int32_t* s, const int32_t* tt, double* C, int64_t ldc, cudaStream_t st);
+// whether the tables have groups that launch_reconstruct16_groups is compiled for
+bool reconstruct16_in_groups(const OzTables& t);
 // shared by the split kernels: shifts of strided vectors (colmax must be zeroed)
 cudaError_t launch_shifts_cols(int bits, int64_t nvec, int64_t len, const double* X, int64_t ld, int32_t* shifts,
                                int32_t* flag, uint64_t* colmax, cudaStream_t st);

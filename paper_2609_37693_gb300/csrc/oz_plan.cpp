@@ -200,10 +200,14 @@ void fill_group_tables(OzTables* tp, const uint32_t* moduli, int Q, const Big& P
 }
 
 // Groups of consecutive moduli for the reconstruct of 16-bit digits: each group
-// takes moduli while its largest sum, (size) M_g, stays below 2^32. Left unset
-// unless the sum of these over the groups stays below 2^32 (each 64-bit limb
-// accumulator then holds), P is below 2^125 and the kernel's table of 32
-// multiples of P covers the sum (below Q P).
+// takes moduli while its largest sum, (size) M_g, stays below kDigit16GroupSum. Left
+// unset unless the sum of these over the groups stays below 2^32 (each 64-bit limb
+// accumulator then holds; with up to eight groups a bound of 2^32 for each would
+// not give it, and 2^30 does for every configuration), P is below 2^125 and the
+// kernel's table of 32 multiples of P covers the sum (below Q P). The kernel is
+// compiled for the sizes that this bound gives (with_sizes in oz_reconstruct.cu):
+// another bound asks for other shapes there, else the plans run in pairs.
+constexpr double kDigit16GroupSum = 1073741824.0;   // 2^30
 void fill_digit16_groups(OzTables* tp, const uint32_t* moduli, int Q, const Big& P) {
   OzTables& t = *tp;
   t.rh_ng = 0;
@@ -214,7 +218,7 @@ void fill_digit16_groups(OzTables* tp, const uint32_t* moduli, int Q, const Big&
     if (ng == OZ_RG_MAX) return;
     uint64_t M = 1;
     int e = q;
-    while (e < Q && (double)(e - q + 1) * (double)M * moduli[e] < 1073741824.0) M *= moduli[e++];
+    while (e < Q && (double)(e - q + 1) * (double)M * moduli[e] < kDigit16GroupSum) M *= moduli[e++];
     if (e == q) return;
     t.rh_start[ng] = q;
     for (int i = q; i < e; ++i) t.rh_w[i] = (uint32_t)(M / moduli[i]);

@@ -1266,6 +1266,10 @@ cudaError_t launch_reconstruct16_groups(const OzTables& T, int64_t m, int64_t n,
   });
 }
 
+bool reconstruct16_in_groups(const OzTables& T) {
+  return T.rh_ng > 0 && with_sizes(T, [](auto) { return cudaSuccess; }) == cudaSuccess;
+}
+
 // Whether the grouped reconstruct of a plan's products takes the groups'
 // kernel (eight entries per thread) rather than the pairs' (four).
 bool reconstruct_grouped_eight(const OzTables& T) { return group_shape(T) >= 0; }

@@ -4,7 +4,8 @@
 // nothing ever arrives, the wait runs out after about 2 s of %globaltimer,
 // records bit 1 in the status word, and the kernel returns, so the context
 // stays usable. No memory but the block's shared memory and the status word
-// is touched.
+// is touched. And a view of the planner's tables: the groups of moduli of the
+// 16-bit-digit reconstruct.
 #include <stdint.h>
 
 #include "oz_internal.h"
@@ -36,4 +37,13 @@ extern "C" oz_status oz_selftest_bounded_wait(int arrive, int32_t* status, void*
   if (!status) return OZ_ERR_INVALID_ARG;
   oz::bounded_wait_kernel<<<1, 32, 0, static_cast<cudaStream_t>(stream)>>>(status, arrive ? 1 : 0);
   return cudaGetLastError() == cudaSuccess ? OZ_OK : OZ_ERR_CUDA;
+}
+
+extern "C" oz_status oz_selftest_digit16_groups(oz_plan plan, int* groups, int* starts, int* compiled) {
+  if (!plan || !plan->is_fp || !groups || !starts || !compiled) return OZ_ERR_INVALID_ARG;
+  const OzTables& T = plan->tab;
+  *groups = T.rh_ng;
+  for (int g = 0; g <= T.rh_ng; ++g) starts[g] = T.rh_ng > 0 ? T.rh_start[g] : 0;
+  *compiled = oz::reconstruct16_in_groups(T) ? 1 : 0;
+  return OZ_OK;
 }
