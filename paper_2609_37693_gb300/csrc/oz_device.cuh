@@ -17,11 +17,12 @@ static __device__ __forceinline__ int32_t shift_from_maxbits(uint64_t mb, int be
   return beta - e;
 }
 
-// Programmatic dependent launch: a kernel launched by launch_pdl (oz_launch.h)
-// may start while the kernel before it on the stream is still running. Every
-// kernel of a product therefore waits here, before its first access to global
-// memory, until that kernel has finished and its writes are visible, and then
-// lets its own successor be scheduled. Both are no-ops after a plain launch.
+// Programmatic dependent launch: a kernel launched dependent (launch_kernel in
+// oz_launch.h, which names these kernels) may start while the kernel before it on
+// the stream is still running. Each of them therefore waits here, before its first
+// access to global memory, until that kernel has finished and its writes are
+// visible, and then lets its own successor be scheduled. Both are no-ops after a
+// plain launch, the only one that kernels without the wait may have.
 static __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 static __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

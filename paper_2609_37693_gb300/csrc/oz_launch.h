@@ -1,8 +1,11 @@
 // oz_launch.h -- kernel launches with programmatic stream serialisation: the
 // kernel may be scheduled while its predecessor on the stream drains, so the
 // launch latency and the set-up of one phase run under the tail of the phase
-// before. The kernels launched this way call pdl_wait (oz_device.cuh) before
-// they touch global memory.
+// before. Only a kernel that calls pdl_wait (oz_device.cuh) before it touches
+// global memory may be launched dependent: the joint splits (split_both_kernel,
+// split_tiles_kernel), the GEMMs of one product (gemm_tc_kernel,
+// gemm_tc_pair_kernel) and reconstruct_groups8_kernel. All others have no wait
+// and are correct in plain stream order only.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -43,12 +46,6 @@ inline cudaError_t launch_kernel(bool dependent, void (*kernel)(KArgs...), dim3 
   }
   cfg.attrs = attr;
   return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
-}
-
-template <typename... KArgs, typename... Args>
-inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
-                              int cluster, Args... args) {
-  return launch_kernel(true, kernel, grid, block, smem, st, cluster, args...);
 }
 
 }  // namespace oz

@@ -846,8 +846,6 @@ __global__ void __launch_bounds__(256, 2) reconstruct_groups_kernel(const __grid
   __shared__ uint32_t buf[2][Q * 256];
   fill_kP<Q>(T, kPs);
   __syncthreads();
-  pdl_wait();
-  pdl_trigger();
   const int tpr = 1 << tpr_log2, rows = 256 >> tpr_log2;
   const int r_in = threadIdx.x >> tpr_log2, c_in = threadIdx.x & (tpr - 1);
   const int64_t plane = m * ldy;
@@ -1161,15 +1159,13 @@ cudaError_t launch_L16(const OzTables& T, int64_t m, int64_t n, const uint16_t* 
   return cudaGetLastError();
 }
 
-// CTAs of a kernel resident per SM, times the SM count (cached per device)
+// CTAs of a kernel resident per SM, times the SM count
 template <typename K>
 int persistent_grid(K kernel, int threads) {
-  static int cache[64][2];                    // [device] = {kernel-independent SM count, CTAs per SM}
   int dev = 0, sms = 0, per = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return 0;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, threads, 0) != cudaSuccess) return 0;
-  (void)cache;
   return sms * (per > 0 ? per : 1);
 }
 
