@@ -595,9 +595,12 @@ static_assert((2 * P_STAGES + 5) * 8 <= kHolderOff, "pair kernel barriers overla
 static_assert((2 * STAGES + 5) * 8 <= kHolderOff, "barriers overlap the TMEM address");
 // Epilogue warps of the pair kernel: sixteen when every unit is one slab (the
 // epilogue then bounds the kernel) and for grouped products; eight for one
-// product of several slabs: 8192^3 products 11.3 ms under the power cap against
-// 11.5 with four or sixteen, 4096^3 1.57 ms with any, 2048^3 GEMMs 170 us
-// against 172 and 169.
+// product of several slabs. Four are the slowest throughout; sixteen are 0.3 to
+// 0.7 % faster than eight from cool, eight 1.1 to 1.3 % faster under the power cap
+// from 8192^3 on. Products with four / eight / sixteen warps: from cool 293 / 283 /
+// 281 us at 2048^3, 1.497 / 1.483 / 1.474 ms at 4096^3, 10.18 / 10.07 / 10.04 at
+// 8192^3; under the cap 1.567 / 1.555 / 1.548, 11.43 / 11.13 / 11.26 and, at
+// 16384^3, 95.0 / 92.5 / 93.7.
 constexpr int kPairEpiWarps = 16;
 constexpr int kPairEpiWarpsMulti = 8;
 

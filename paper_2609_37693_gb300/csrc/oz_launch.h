@@ -13,12 +13,21 @@
 
 namespace oz {
 
-// Outputs from this many entries on are launched in plain stream order. A
-// dependent launch is worth 2 us at 2048^3 (285 against 287) and most of the
-// gaps of a small product, but cost a larger one more than that: 2400 x 2400 x
-// 512 200 us against 191, 3000 x 2500 x 2000 507 against 499, 65536 x 256 x 256
-// 390 us against 382, 8192 x 8192 x 256 1001 against 978, 16384^3 94.9 ms
-// against 94.3.
+// Outputs from this many entries on are launched in plain stream order. What
+// a dependent launch costs them is the reconstruct's L1: its blocks start on SMs
+// that still hold a GEMM block, so they keep that block's split of the SM's memory,
+// nearly all of it shared, where a plain launch gives L1 the larger part. At
+// 2400^2 the reconstruct takes 61.7 us, and 78.1 launched plain with all memory asked
+// for as shared; at 4096^2 99 and 114. The gaps that the two dependent launches hide
+// are worth a few microseconds whatever the size, so the line lies where the two
+// together stop gaining, between 4 Mi entries (1.5 us gained) and 5.8 Mi (12 lost).
+// Products, us, both plain / GEMM dependent / reconstruct dependent / both:
+//   1024 x 1024 x 1024   78.4   75.9   73.9   70.7
+//   2048 x 2048 x 2048    285    282    286    283
+//   2400 x 2400 x 512     184    182    198    196
+//   3000 x 2500 x 2000    491    487    506    503
+//   65536 x 256 x 256     371    368    381    379
+//   8192 x 8192 x 256     934    931    982    977
 constexpr int64_t kDependentMaxOutput = 5ll << 20;
 
 // Whether the GEMM and the reconstruct of an m x n output are launched dependent.

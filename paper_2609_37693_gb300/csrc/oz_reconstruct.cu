@@ -562,8 +562,9 @@ __device__ __forceinline__ void multiple_of_P(const uint4* kP, int q, uint32_t (
 // at 4096^2, us: no moves here, one move for every entry, and as it is now):
 //   Q = 16, phi 0.5    103  110   99      Q = 9, phi 0.5        248  331   93
 //   Q = 16, phi 4      155  110  101      Q = 16, all subnormal 298  382  125
-//   Q = 12, phi 0.5    268   96   95      E4M3, all subnormal   199  394  162
-// (E4M3's 199: moduli in pairs, every entry on the general path.)
+//   Q = 12, phi 0.5    268   96   95
+// E4M3, all subnormal: 162, 394 when they are recomputed from the digits, 199 with
+// moduli in pairs.
 template <int L>
 __device__ __forceinline__ uint32_t round4_fast(const uint4* kP, int kmax, const uint32_t (&S)[4][L],
                                                 const float (&f)[4], int (&ex)[4], uint64_t (&out)[4]) {
