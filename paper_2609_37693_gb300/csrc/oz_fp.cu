@@ -429,7 +429,10 @@ __global__ void __launch_bounds__(256, 3) split_fp_rows_tab_kernel(const __grid_
 // turn with one barrier per channel, and leave as whole rows: stored straight
 // from the lanes that hold them they went out in pieces of 32 or 16 bytes, which
 // bound the kernel (E2M1 494 us at 4096^2).
-constexpr int kFpTableMax = 48 * 1024;                                   // bytes of a plan's code table
+// Bytes of a plan's code table: with the row split's own shared memory (72 bytes)
+// it has to stay within the 48 KB that a launch gets without asking for more (every
+// base configuration: 6 to 27 KB).
+constexpr int kFpTableMax = 47 * 1024;
 constexpr int kFpColThreads = 512, kFpColTileH = 128;
 constexpr int kFpStagePitch = 144, kFpStagePlane = 32 * kFpStagePitch;   // bytes
 

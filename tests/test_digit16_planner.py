@@ -3,6 +3,8 @@ reconstruct: for every frozen base configuration they cover the moduli in order,
 keep the bounds of the kernel's 32- and 64-bit sums, and have sizes that the kernel
 is compiled for, so that no configuration falls back to pairs unseen."""
 import math
+import pathlib
+import re
 
 import pytest
 
@@ -52,3 +54,19 @@ def test_widened_and_integer_plans():
     plan = oz.PlanFP("E4M3", 16384, 69)
     assert oz.oz_selftest_digit16_groups(plan.handle) == (oz.OZ_OK, [0], False)
     assert oz.oz_selftest_digit16_groups(oz.Plan(16, 0, 64).handle)[0] == oz.OZ_ERR_INVALID_ARG
+
+
+def test_code_tables_fit_the_row_split():
+    """The split's table (a word per balanced residue) and the kernel's own shared
+    memory stay within the 48 KB of a launch that asks for no more, at the
+    limit that the launcher allows and for every base configuration."""
+    src = (pathlib.Path(oz.__file__).parent / "csrc" / "oz_fp.cu").read_text()
+    limit = int(re.search(r"kFpTableMax = (\d+) \* 1024;", src).group(1)) * 1024
+    own = 8 * 8 + 4                                       # red[8], s_sh
+    assert limit + own <= 48 * 1024 - 256
+    for fmt, k in CONFIGS:
+        try:
+            moduli = oz.PlanFP(fmt, k).moduli
+        except oz.OzError:
+            continue
+        assert sum(2 * (m // 2) + 1 for m in moduli) * 4 <= limit
